@@ -66,12 +66,13 @@ typedef enum {
     /* FP64 arithmetic: FP64 tensor-core MMA (mma.sync f64) with FP64 accumulation.  For
        FP32-stored operands the values are widened exactly and the result rounded once. */
     COMET_PREC_NATIVE = 0,
-    /* Split precision: each operand is scaled by 2^-e (e = exponent of its largest magnitude)
-       and every element split into three bfloat16 fixed-point parts, x * 2^-e rounded to
-       nearest on the grids 2^-6, 2^-14 and 2^-22; six of the nine part products (hh, hm, mh,
-       hl, lh, mm) run on the tensor cores with FP32 accumulation, the hh products in chunks of
-       up to 1024 K values that sum exactly.  Target: normwise relative error <= 1e-6 against
-       FP64 (measured 3.4e-7 on the o=64 v=192 workload). */
+    /* Split precision (the name is historical): each operand is scaled by a power of two taken
+       from its largest magnitude and every element split into two FP16 parts, the nearest FP16
+       value and the nearest one to what is left; three of the four part products (hh, hl, lh) run
+       on the tensor cores with FP32 accumulation in chunks of 32 or 64 K values, which are added in
+       FP32.  Target: normwise relative error <= 1e-6 against FP64 (measured 1.6e-7 on the o=64
+       v=192 workload).  Batched plans split into three fixed-point bfloat16 parts and keep six
+       products. */
     COMET_PREC_SPLIT_BF16 = 1,
     /* FP64 emulated on the BF16 tensor cores (FP64 storage only, else COMET_ERR_DTYPE): each
        operand is scaled by 2^-e and written as six integer-valued bfloat16 slices on the grids
@@ -101,8 +102,8 @@ typedef struct {
     size_t workspace_cap;       /* 0 = unlimited; intermediates above it are refused */
     int form;                   /* -1 = planner's choice; k >= 0 = k-th enumerated TTGT form
                                    of every binary step (for the permutation ablation) */
-    int64_t kc;                 /* split path: K elements per FP32 accumulation chunk before
-                                   the chunk is added into the compensated sum (0 = whole K) */
+    int64_t kc;                 /* split path: an upper limit of the K elements per accumulation
+                                   chunk; the kernel's chunks are 32 or 64 whatever its value */
     int64_t timeout_ms;         /* device-side wait limit; 0 = default (2000 ms) */
     int debug_flags;            /* bit 0: withhold one operand load in the split GEMM so that
                                    its wait runs out (fault-injection test); bit 3, builds with

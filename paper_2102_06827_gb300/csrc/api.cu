@@ -274,7 +274,7 @@ static comet_status_t run_plan(const Plan &P, const void *const *inputs, void *o
             XposeParams xa = st.pre_a, xb = st.pre_b;
             xa.in = g.A; xa.out = w + st.ws_parts_a; xa.scale_bits = sc_a;
             xb.in = g.B; xb.out = w + st.ws_parts_b; xb.scale_bits = sc_b;
-            const int64_t n_planes = st.kernel == KK_GEMM_EMU ? 6 : 3;
+            const int64_t n_planes = st.kernel == KK_GEMM_EMU ? 6 : 2;
             xa.dbg_in = g.dbg_a; xa.dbg_out = dbg_range(xa.out, n_planes * xa.out_plane * 2);
             xb.dbg_in = g.dbg_b; xb.dbg_out = dbg_range(xb.out, n_planes * xb.out_plane * 2);
             xa.status = xb.status = status;
@@ -298,7 +298,7 @@ static comet_status_t run_plan(const Plan &P, const void *const *inputs, void *o
             } else {
                 ProfScope ps(PK_SPLIT, stream);
                 e = launch_gemm_split(g, w + st.ws_parts_a, w + st.ws_parts_b, st.kpad, sc_a, sc_b,
-                                      P.opts.kc, es, P.opts.debug_flags, stream, 0, st.ksplit,
+                                      es, P.opts.debug_flags, stream, st.want_ksplit,
                                       reinterpret_cast<float *>(w + st.ws_ksplit), (int64_t)st.ksplit_bytes);
                 if (e != cudaSuccess) return cuda_status(e, "split gemm kernel");
             }
@@ -391,7 +391,7 @@ static comet_status_t run_host_pipe(const Plan &P, int n_calls, const void *cons
     char *parts_x0 = w + (x_is_b ? st.ws_parts_b : st.ws_parts_a);
     char *parts_w0 = w + (x_is_b ? st.ws_parts_a : st.ws_parts_b);
     const bool emu = st.kernel == KK_GEMM_EMU;
-    const size_t n_planes = emu ? 6 : 3;
+    const size_t n_planes = emu ? 6 : 2;
     // every slice's planes sit after those of the slices before it
     auto parts_x = [&](int j) { return parts_x0 + n_planes * (size_t)(h.rows_inner * h.xb[j]) * (size_t)st.kpad * 2; };
     auto parts_w = [&](int i) { return parts_w0 + n_planes * (size_t)(h.w_rows_inner * h.wb[i]) * (size_t)st.kpad * 2; };
@@ -546,8 +546,9 @@ static comet_status_t run_host_pipe(const Plan &P, int n_calls, const void *cons
                 e = launch_gemm_emu(g, pa, pb, st.kpad, sa, sb, P.opts.debug_flags, s, 0);
             } else {
                 ProfScope ps(PK_SPLIT, s);
-                e = launch_gemm_split(g, pa, pb, st.kpad, sa, sb, P.opts.kc, (int)es, P.opts.debug_flags, s, 0,
-                                      st.ksplit, reinterpret_cast<float *>(w + st.ws_ksplit), (int64_t)st.ksplit_bytes);
+                e = launch_gemm_split(g, pa, pb, st.kpad, sa, sb, (int)es, P.opts.debug_flags, s,
+                                      st.want_ksplit, reinterpret_cast<float *>(w + st.ws_ksplit),
+                                      (int64_t)st.ksplit_bytes);
             }
             if (e != cudaSuccess) return cuda_status(e, "host pipeline gemm");
             if (h.blockwise) {   // this block's result back as soon as it is done

@@ -9,7 +9,7 @@
 // registers.  The same engine performs three element operations:
 //   OP_MOVE   raw 4/8-byte words (bit-exact permutation, comet_transpose)
 //   OP_SCALE  out = alpha * in (+ beta * out)  (ta.copy with alpha)
-//   OP_SPLIT  x -> three bfloat16 planes hi, mid, lo (split pre-pass of the split-BF16 GEMM)
+//   OP_SPLIT  x -> two FP16 planes h, l (split pre-pass of the split GEMM)
 //   OP_SPLIT6 FP64 x -> six integer-valued bfloat16 planes (pre-pass of the FP64 emulation)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -32,8 +32,19 @@ struct alignas(sizeof(T) * N) Vec {
     T v[N];
 };
 
+// scale of a pre-pass: the operand's exponent (OP_SPLIT6) and 2^(14-e) as two factors (OP_SPLIT)
+template <int OP, typename T>
+struct OpScale {
+    int e = 0;
+    T s0 = 1, s1 = 1;
+    __device__ __forceinline__ explicit OpScale(const XposeParams &p) {
+        if constexpr (OP == OP_SPLIT || OP == OP_SPLIT6) e = scale_exponent<T>(p.scale_bits);
+        if constexpr (OP == OP_SPLIT) half_scales<T>(e, s0, s1);
+    }
+};
+
 template <int OP, typename T, int VO>
-__device__ __forceinline__ void emit(const XposeParams &p, int64_t off, const T (&x)[VO], int e) {
+__device__ __forceinline__ void emit(const XposeParams &p, int64_t off, const T (&x)[VO], const OpScale<OP, T> &e) {
 #ifdef COMET_DEBUG
     if (p.plant && blockIdx.x == 0 && threadIdx.x == 0) off += p.plant;   // test of the range check
 #endif
@@ -58,21 +69,20 @@ __device__ __forceinline__ void emit(const XposeParams &p, int64_t off, const T 
         }
         *reinterpret_cast<Vec<VO, T> *>(o) = w;
     } else if constexpr (OP == OP_SPLIT) {
-        Vec<VO, __nv_bfloat16> h, m, l;
+        Vec<VO, __half> h, l;
 #pragma unroll
-        for (int q = 0; q < VO; ++q) split3<T>(x[q], e, h.v[q], m.v[q], l.v[q]);
-        __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(p.out) + off;
-        if (!dbg_ok(p.dbg_out, o, 2 * (2 * p.out_plane + VO), p.status)) return;   // all three planes
-        *reinterpret_cast<Vec<VO, __nv_bfloat16> *>(o) = h;
-        *reinterpret_cast<Vec<VO, __nv_bfloat16> *>(o + p.out_plane) = m;
-        *reinterpret_cast<Vec<VO, __nv_bfloat16> *>(o + 2 * p.out_plane) = l;
+        for (int q = 0; q < VO; ++q) split2<T>(x[q], e.s0, e.s1, h.v[q], l.v[q]);
+        __half *o = reinterpret_cast<__half *>(p.out) + off;
+        if (!dbg_ok(p.dbg_out, o, 2 * (p.out_plane + VO), p.status)) return;   // both planes
+        *reinterpret_cast<Vec<VO, __half> *>(o) = h;
+        *reinterpret_cast<Vec<VO, __half> *>(o + p.out_plane) = l;
     } else {
         static_assert(sizeof(T) == 8, "the six-way split is for FP64 operands");
         Vec<VO, __nv_bfloat16> sl[6];
 #pragma unroll
         for (int q = 0; q < VO; ++q) {
             __nv_bfloat16 v[6];
-            split6((double)x[q], e, v);
+            split6((double)x[q], e.e, v);
 #pragma unroll
             for (int k = 0; k < 6; ++k) sl[k].v[q] = v[k];
         }
@@ -145,7 +155,7 @@ __global__ void __launch_bounds__(XT, 8) xpose_tile_kernel(const XposeParams p) 
         out_row[r] = ro;
     }
     __syncthreads();
-    const int e = (OP == OP_SPLIT || OP == OP_SPLIT6) ? scale_exponent<T>(p.scale_bits) : 0;
+    const OpScale<OP, T> e(p);
     {   // loads: p.ll threads per row, each with a fixed u; batches of rows in flight together
         const uint32_t lanes = p.ll, rpp = p.rpp_l;
         const uint32_t r0 = fd_div(t, p.fd_ll);
@@ -233,7 +243,7 @@ __global__ void __launch_bounds__(XT, 6) xpose_copy_kernel(const XposeParams p) 
     }
     __syncthreads();
     const T *__restrict__ in = reinterpret_cast<const T *>(p.in);
-    const int e = (OP == OP_SPLIT || OP == OP_SPLIT6) ? scale_exponent<T>(p.scale_bits) : 0;
+    const OpScale<OP, T> e(p);
     constexpr int UB = VW * sizeof(T) >= 16 ? 4 : 8;
     const uint32_t lanes = p.ll;
     const uint32_t rpp = p.rpp_l;
@@ -306,7 +316,7 @@ __global__ void __launch_bounds__(XT) xpose_run_kernel(const XposeParams p) {
     const uint32_t nu = min(tu, p.u.total - u0);
     const int64_t su = p.u.s0[0], so = p.u.s1[0];
     const T *__restrict__ in = reinterpret_cast<const T *>(p.in);
-    const int e = (OP == OP_SPLIT || OP == OP_SPLIT6) ? scale_exponent<T>(p.scale_bits) : 0;
+    const OpScale<OP, T> e(p);
     constexpr int UB = VW * sizeof(T) >= 16 ? 4 : 8;
     const int64_t ri = (int64_t)u0 * su, ro = (int64_t)u0 * so;
     const uint32_t nvec = nu / VW * VW;
@@ -527,7 +537,7 @@ cudaError_t launch_scale(const XposeParams &p, int elem_bytes, int vi, int vo, c
     return launch_op<OP_SCALE, double>(p, vi, vo, s);
 }
 
-// The split pre-pass writes bfloat16 planes; its store vectors hold as many bf16 as the input
+// The split pre-pass writes FP16 planes; its store vectors hold as many FP16 as the input
 // vector holds input elements (4 for FP32, 2 for FP64), which keeps every plane's stores
 // aligned whenever the input-width condition holds for the output strides and the plane stride.
 cudaError_t launch_split(const XposeParams &p, int elem_bytes, int vi, int vo, cudaStream_t s) {

@@ -16,6 +16,8 @@
 #include <set>
 #include <sstream>
 
+#include "split_schedule.h"
+
 namespace comet {
 
 // Machine constants of the cost model (GB300): HBM copy bandwidth and dense tensor-core and
@@ -393,9 +395,9 @@ std::vector<std::vector<int>> group_orders(const std::vector<int> &g,
     return res;
 }
 
-// modelled time of one form of a binary step
+// modelled time of one form of a binary step (t_split: the split GEMM's own modelled time)
 void cost_form(const Plan &P, const std::vector<int> &lx, const std::vector<int> &ly,
-               const std::vector<int> &lz, bool z_free_layout, int kernel, Form *f) {
+               const std::vector<int> &lz, bool z_free_layout, int kernel, double t_split, Form *f) {
     const std::vector<int64_t> &ext = P.extent;
     double es = (double)dtype_size(P.dtype);
     const std::vector<int> &lm = f->swap ? ly : lx;   // M operand labels
@@ -409,10 +411,10 @@ void cost_form(const Plan &P, const std::vector<int> &lx, const std::vector<int>
     f->eff_store = run_eff(std::min(run_c, 32.0) * es * 2);
     double t_store = M * N * es / (kHbmBytesPerS * f->eff_store);
     if (kernel == KK_GEMM_SPLIT || kernel == KK_GEMM_EMU) {
-        // pre-passes: read the operand, write 3 (split) or 6 (emulated FP64) bf16 planes in
+        // pre-passes: read the operand, write 2 FP16 (split) or 6 bf16 (emulated FP64) planes in
         // [rows][K] order; the transpose engine's efficiency follows from the runs on both sides
         const bool emu = kernel == KK_GEMM_EMU;
-        const double plane_bytes = emu ? 12.0 : 6.0;
+        const double plane_bytes = emu ? 12.0 : 4.0;
         auto pre = [&](const std::vector<int> &lop, const std::vector<int> &rows, double *eff_out) {
             std::vector<int64_t> e, si, so;
             auto st = label_strides(lop, ext);
@@ -438,9 +440,9 @@ void cost_form(const Plan &P, const std::vector<int> &lx, const std::vector<int>
         double bx = pre(lm, f->M, &f->eff_a), by = pre(ln, f->N, &f->eff_b);
         f->pre_bytes = bx + by;
         double t_pre = bx / (kHbmBytesPerS * f->eff_a) + by / (kHbmBytesPerS * f->eff_b) + 2 * kLaunchS;
-        const double bn = emu ? 80.0 : 256.0, products = emu ? 21.0 : 6.0;
-        double waste = (std::ceil(M / 128) * 128 * std::ceil(N / bn) * bn) / (M * N);
-        double t_mma = products * 2.0 * M * N * K * waste / kBf16FlopsPerS;
+        const double waste = (std::ceil(M / 128) * 128 * std::ceil(N / 80) * 80) / (M * N);
+        const double t_mma = emu ? 21.0 * 2.0 * M * N * K * waste / kBf16FlopsPerS
+                                 : t_split;
         // the epilogue's stores overlap the next tile's main loop, but scattered stores still
         // cost DRAM bandwidth: charge a share of them beyond the overlap
         f->cost = t_pre + std::max(t_mma, t_store) + 0.25 * t_store + kLaunchS;
@@ -523,15 +525,15 @@ void setup_host_pipe(Plan *P, int64_t es, int want, int want_w) {
     h.wc_inner = tc[h.w_label];
     h.w_rows_inner = prod_ext(P->extent, wrows) / h.w_ext;
     const bool emu = st.kernel == KK_GEMM_EMU;
-    const int64_t tm = 128, tn = emu ? 80 : 256;          // output tile of the GEMM kernel
-    const double prods = emu ? 21.0 / 0.6 : 6.0;             // bf16 products per tile (emu: drain-bound)
-    const double t_tile = 2.0 * tm * tn * (double)st.kpad * prods / (kBf16FlopsPerS / 152);
+    const int64_t tm = 128, tn = 80;                      // output tile of the emulated GEMM kernel
+    const double t_tile = 2.0 * tm * tn * (double)st.kpad * (21.0 / 0.6) / (kBf16FlopsPerS / 152);   // drain-bound
     const double bw_in = 200e9, bw_out = 180e9, t_slice = 20e-6;
-    const double planes = emu ? 12.0 : 6.0;
+    const double planes = emu ? 12.0 : 4.0;
     const bool layout_blocks = h.wc_inner * h.w_ext == h.c_inner || h.c_inner * h.ext == h.wc_inner;
-    auto tiles_of = [&](int64_t lx, int64_t lw) {
-        const int64_t r = h.rows_inner * lx, rw = h.w_rows_inner * lw;
-        return h.side ? ((rw + tm - 1) / tm) * ((r + tn - 1) / tn) : ((r + tm - 1) / tm) * ((rw + tn - 1) / tn);
+    auto t_block = [&](int64_t lx, int64_t lw) {   // one GEMM block of lx x lw label indices
+        const int64_t r = h.rows_inner * lx, rw = h.w_rows_inner * lw, M = h.side ? rw : r, N = h.side ? r : rw;
+        return emu ? (double)((((M + tm - 1) / tm) * ((N + tn - 1) / tn) + 151) / 152) * t_tile
+                   : 1e-6 * split_schedule((uint64_t)M, (uint64_t)N, (uint64_t)st.kpad, 76, 1, 0).us;
     };
     const int64_t xu = h.x_inner * h.x_outer, wu = h.w_inner * h.w_outer;
     // slice boundaries: n slices, the first one 1/ramp of an equal slice, the rest equal (the
@@ -592,12 +594,20 @@ void setup_host_pipe(Plan *P, int64_t es, int want, int want_w) {
         const bool sliced = nx > 1 || nw > 1;
         std::vector<char> px(nx, 0), pw(nw, 0);
         std::vector<int> left(nx, nw);
+        // block times: slices of one length share them (a slicing has at most three lengths a side)
+        int ux[32], uw[32];   // nx + nw <= 31 and nx * nw <= 64 for every candidate
+        double tb[64];
+        for (int j = 0; j < nx; ++j) { ux[j] = 0; while (lx(ux[j]) != lx(j)) ++ux[j]; }
+        for (int i = 0; i < nw; ++i) { uw[i] = 0; while (lw(uw[i]) != lw(i)) ++uw[i]; }
+        for (int q = 0; q < nx * nw; ++q) tb[q] = -1.0;
         double t = 0, out = 0;
         for (int u : sd.blocks) {
             const int i = u / nx, j = u % nx;
             if (!pw[i]) { t = std::max(t, rw[i]) + wbytes(i) / es * (es + planes) / kHbmBytesPerS; pw[i] = 1; }
             if (!px[j]) { t = std::max(t, rx[j]) + xbytes(j) / es * (es + planes) / kHbmBytesPerS; px[j] = 1; }
-            t += (double)((tiles_of(lx(j), lw(i)) + 151) / 152) * t_tile + (sliced ? t_slice : 0);
+            double &t_uv = tb[uw[i] * nx + ux[j]];
+            if (t_uv < 0) t_uv = t_block(lx(j), lw(i));
+            t += t_uv + (sliced ? t_slice : 0);
             if (sd.blockwise) out = std::max(out, t) + cbytes(j) * (double)lw(i) / (double)h.w_ext / bw_out;
             else if (--left[j] == 0) out = std::max(out, t) + cbytes(j) / bw_out;
         }
@@ -990,12 +1000,15 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
         for (int swap = 0; swap < 2; ++swap) {
             const std::vector<int> &gm = swap ? J : I, &gn = swap ? I : J;
             const std::vector<int> &lm = swap ? sb.labels : sa.labels, &ln = swap ? sa.labels : sb.labels;
+            const double t_split = kernel != KK_GEMM_SPLIT ? 0.0 : 1e-6 * split_schedule(
+                (uint64_t)prod_ext(P->extent, gm), (uint64_t)prod_ext(P->extent, gn), (uint64_t)prod_ext(P->extent, K),
+                76, 0, 64 << 20).us;
             auto om = group_orders(gm, {&sc.labels, &lm});
             auto on = group_orders(gn, {&sc.labels, &ln});
             auto ok = group_orders(K, {&lm, &ln});
             for (auto &m : om) for (auto &nn : on) for (auto &k : ok) {
                 Form f; f.swap = swap; f.M = m; f.N = nn; f.K = k; f.Bt = Bt;
-                cost_form(*P, sa.labels, sb.labels, sc.labels, free_layout, kernel, &f);
+                cost_form(*P, sa.labels, sb.labels, sc.labels, free_layout, kernel, t_split, &f);
                 forms.push_back(f);
                 if (forms.size() > 20000) break;
             }
@@ -1042,38 +1055,36 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
         int64_t Kx = prod_ext(P->extent, st.form.K);
         st.kpad = (Kx + 7) / 8 * 8;
         int64_t rows_a = prod_ext(P->extent, st.form.M), rows_b = prod_ext(P->extent, st.form.N);
-        const size_t planes = st.kernel == KK_GEMM_EMU ? 6 : 3;
+        const size_t planes = st.kernel == KK_GEMM_EMU ? 6 : 2;
         size_t ba = align(planes * rows_a * st.kpad * 2), bb = align(planes * rows_b * st.kpad * 2);
         st.ws_parts_a = parts_base;
         st.ws_parts_b = parts_base + ba;
-        // K slices: a split GEMM with fewer output tiles than SMs spreads K over more work items
-        // (slices of at least 256 K values, partials at most 256 MB)
-        st.ksplit = 1;
-        if (st.kernel == KK_GEMM_SPLIT && opts.ksplit != 1) {
-            const int64_t tiles = ((rows_a + 127) / 128) * ((rows_b + 255) / 256);
-            const int64_t nkb = (Kx + 31) / 32;
-            int64_t k = opts.ksplit > 1 ? opts.ksplit
-                                        : std::min<int64_t>({(152 + tiles - 1) / tiles, nkb / 8, 16});
-            while (k > 1 && (double)k * tiles * 128 * 256 * 4 > 256.0 * (1 << 20)) --k;
-            st.ksplit = (uint32_t)std::max<int64_t>(1, std::min<int64_t>(k, nkb));
+        size_t bk = 0, least = 0;
+        if (st.kernel == KK_GEMM_SPLIT) {
+            // tile width and K slices (split_schedule).  The partial sums stay inside the library's
+            // static scratch when the plan without them would (three planes per operand were
+            // kept before; the step's room is never less than theirs), else within 256 MB
+            least = align((size_t)6 * rows_a * st.kpad) + align((size_t)6 * rows_b * st.kpad);
+            const int64_t fixed = COMET_NOALLOC_MAX_BYTES - 256;
+            const int64_t limit = (int64_t)(parts_base + least) <= fixed ? fixed - (int64_t)(parts_base + ba + bb)
+                                                                         : (int64_t)256 << 20;
+            st.want_ksplit = opts.ksplit > 0 ? (uint32_t)opts.ksplit : 0;
+            const SplitSchedule sch = split_schedule((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, 76,
+                                                     st.want_ksplit, limit / 256 * 256);
+            st.ksplit = sch.ksplit;
+            st.tile_n = sch.bn;
+            bk = (size_t)split_partial_bytes((uint64_t)rows_a, (uint64_t)rows_b, sch);
+            const int64_t tiles = ((rows_a + 127) / 128) * ((rows_b + 255) / 256), tail = tiles % 152;
+            st.tail_tiles = 0;
+            st.tail_slices = 1;
+            if (st.ksplit == 1 && tiles > 152 && tail > 0 && 2 * tail <= 152) {
+                st.tail_tiles = (uint32_t)tail;
+                st.tail_slices = (uint32_t)std::min<int64_t>({4, 152 / tail, (Kx + 31) / 32});
+            }
         }
         st.ws_ksplit = parts_base + ba + bb;
-        // partials: every tile's K slices (128 x 256 floats per tile and slice), or with whole-K
-        // tiles the slices of a partial last wave over 152 SMs (at most 152 tile slices)
-        const int64_t tiles = ((rows_a + 127) / 128) * ((rows_b + 255) / 256);
-        size_t bk = 0;
-        if (st.ksplit > 1) bk = (size_t)st.ksplit * tiles * 128 * 256 * 4;
-        else if (st.kernel == KK_GEMM_SPLIT && tiles > 152) bk = (size_t)152 * 128 * 256 * 4;
-        // the launch's tail rule on a 152-SM GB300 (it applies the rule to the device's own count)
-        st.tail_tiles = 0;
-        st.tail_slices = 1;
-        if (st.kernel == KK_GEMM_SPLIT && st.ksplit == 1 && tiles > 152 && tiles % 152 != 0 &&
-            2 * (tiles % 152) <= 152) {
-            st.tail_tiles = (uint32_t)(tiles % 152);
-            st.tail_slices = (uint32_t)std::min<int64_t>({4, 152 / (tiles % 152), (Kx + 31) / 32});
-        }
         st.ksplit_bytes = bk;
-        parts_max = std::max(parts_max, ba + bb + align(bk));
+        parts_max = std::max(parts_max, std::max(least, ba + bb + align(bk)));
     }
     for (auto &st : P->steps) {
         if (st.kernel == KK_REDUCE) {   // y[kept] = sum over the private labels of the operand
@@ -1263,7 +1274,7 @@ std::string describe_plan(const Plan &P) {
               << ",\"n_forms\":" << s.n_forms << ",\"form_index\":" << s.form_index
               << ",\"cost_s\":" << s.form.cost << ",\"pre_bytes\":" << s.form.pre_bytes
               << ",\"eff_store\":" << s.form.eff_store << ",\"flops\":" << s.flops
-              << ",\"ksplit\":" << s.ksplit;
+              << ",\"ksplit\":" << s.ksplit << ",\"tile_n\":" << s.tile_n;
             if (s.kernel == KK_GEMM_SPLIT)
                 o << ",\"tail_tiles\":" << s.tail_tiles << ",\"tail_slices\":" << s.tail_slices;
         }

@@ -68,15 +68,18 @@ struct Step {
     int form_index = 0;
     double flops = 0;
     bool final_step = false;
-    // split path workspace for the bf16 parts: [3][rows][kpad]
+    // split path workspace for the parts: [2][rows][kpad] FP16 (split) or [6][rows][kpad] bf16 (emulated)
     size_t ws_parts_a = 0, ws_parts_b = 0;
     size_t ws_scales = 0;        // two 8-byte words: max |A|, max |B| of the step's operands
     int64_t kpad = 0;
-    uint32_t ksplit = 1;         // split GEMM: K slices per output tile
+    uint32_t want_ksplit = 0;    // split GEMM: the caller's K slices (0 = free)
+    uint32_t ksplit = 1, tile_n = 0;   // split GEMM: K slices and tile width on 152 SMs (the launch
+                                       // makes the same choice from the device's own count)
     size_t ws_ksplit = 0;        // workspace offset of the slices' FP32 partials
-    size_t ksplit_bytes = 0;     // their size (K slices of every tile, or of a partial last wave)
-    uint32_t tail_tiles = 0, tail_slices = 1;   // whole-K split GEMM on 152 SMs: the partial last
-                                                // wave's tiles and their K slices (1 = no tail split)
+    size_t ksplit_bytes = 0;     // their size
+    uint32_t tail_tiles = 0, tail_slices = 1;   // description: what 128 x 256 tiles leave over after
+                                                // whole waves of 152 SMs, at most half of them, and
+                                                // the K slices of it that would fill them
     // precomputed parameter blocks (pointers filled at launch)
     GemmParams gemm;             // for both GEMM kernels (offsets in elements)
     XposeParams pre_a, pre_b;    // split pre-passes (A then B operand)

@@ -1,6 +1,7 @@
 // Fixed-point bfloat16 splits shared by the split pre-passes and the batched kernels.
 #pragma once
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 namespace comet {
@@ -35,6 +36,28 @@ __device__ __forceinline__ void split3(T x, int e, __nv_bfloat16 &h, __nv_bfloat
         m = __float2bfloat16_rn((float)fm);
         l = __float2bfloat16_rn((float)fl);
     }
+}
+
+// Two-part FP16 split of the split GEMM's pre-pass: x 2^(14-e) = h + l up to half a unit of l, h
+// and l each the nearest FP16 value to what is left (kHalfShift = 14 puts the operand's largest
+// magnitude into [2^14, 2^15), so that the exponent range of FP16 lies below it).  The residual
+// x' - h is exact in the input precision and at most half a unit of h; what remains after l is at
+// most 2^-23 of the power of two below |x'| (never more than split3 leaves), or 2^-25 where l is
+// subnormal.  `s0`, `s1`: 2^(14-e) as a product of two powers of two, each inside the type's range.
+constexpr int kHalfShift = 14;
+
+template <typename T>
+__device__ __forceinline__ void half_scales(int e, T &s0, T &s1) {
+    const int s = kHalfShift - e, a = s / 2;
+    if constexpr (sizeof(T) == 4) { s0 = ldexpf(1.0f, a); s1 = ldexpf(1.0f, s - a); }
+    else { s0 = ldexp(1.0, a); s1 = ldexp(1.0, s - a); }
+}
+
+template <typename T>
+__device__ __forceinline__ void split2(T x, T s0, T s1, __half &h, __half &l) {
+    const T xs = x * s0 * s1;
+    h = __float2half_rn((float)xs);
+    l = __float2half_rn((float)(xs - (T)__half2float(h)));
 }
 
 // Fixed-point six-way split of an FP64 value (the FP64-emulation pre-pass): x' = x 2^-e

@@ -1,0 +1,74 @@
+// Tile width and K slicing of the split GEMM, chosen from the GEMM's sizes.  Shared by the
+// planner (which sizes the partial sums' workspace) and the launcher.
+#pragma once
+#include <stdint.h>
+
+#include <algorithm>
+
+namespace comet {
+
+constexpr int kSplitBM = 256;     // output rows per CTA pair
+constexpr int kSplitBK = 64;      // K values per shared-memory stage
+constexpr int kSplitMaxBN = 192;  // output columns per CTA pair: 48, 96, 144, 192
+
+struct SplitSchedule {
+    uint32_t bn = kSplitMaxBN;    // output columns per pair
+    uint32_t ksplit = 1;          // K slices per output tile (FP32 partials when above 1)
+    double us = 0;                // modelled time
+};
+
+// Accumulation of a K slice of `stages` stages: K steps of 16 values per chunk in tensor memory (which
+// truncates: short chunks lose less, but each costs a drain) and chunks per first-level sum of
+// the epilogue (about the square root of the chunks, so that neither level adds many terms).
+inline void split_chunks(uint32_t stages, uint32_t *steps, uint32_t *group) {
+    // 32 values up to K = 4096 (12 % more of the GEMM's time at 1633^3, error 1.43 -> 1.23e-7), 64 beyond
+    // (8.6 against 7.7 ms at 12288^3, where the sums' own rounding is as large)
+    *steps = stages <= 64 ? 2 : 4;
+    const uint32_t n = stages * (4 / *steps);
+    uint32_t g = 1;
+    while (g * g < n) ++g;
+    *group = g;
+}
+
+// bytes of the FP32 partial sums of a schedule
+inline int64_t split_partial_bytes(uint64_t M, uint64_t N, const SplitSchedule &s) {
+    if (s.ksplit <= 1) return 0;
+    const int64_t tiles = (int64_t)((M + kSplitBM - 1) / kSplitBM) * (int64_t)((N + s.bn - 1) / s.bn);
+    return tiles * s.ksplit * kSplitBM * s.bn * 4;
+}
+
+// The schedule with the least modelled time over the tile widths and K slices whose partial
+// sums fit `partial_limit` bytes.  want_ksplit: 0 = free, k = as near to k slices as K allows.
+// The model, at 1.9 GHz: a pair's stage of 64 K values takes 6 * bn cycles of MMA, but not less
+// than 1000 (its loads: (128 + bn/2) * 256 bytes per SM at what the L2 gives all SMs together); a tile
+// takes 5000 + 10 * bn cycles around its main loop (pipeline fill, last drain, stores); K slices
+// add a launch and their partial sums' traffic.
+inline SplitSchedule split_schedule(uint64_t M, uint64_t N, uint64_t K, uint32_t pairs, uint32_t want_ksplit,
+                                    int64_t partial_limit) {
+    const uint64_t mt = (M + kSplitBM - 1) / kSplitBM;
+    const uint32_t nch = (uint32_t)std::max<uint64_t>(1, (K + kSplitBK - 1) / kSplitBK);
+    SplitSchedule best;
+    bool have = false;
+    for (uint32_t bn = 48; bn <= (uint32_t)kSplitMaxBN; bn += 48) {
+        const uint64_t tiles = mt * ((N + bn - 1) / bn);
+        const double chunk = std::max(6.0 * bn, std::max(1000.0, (128 + bn / 2) * 256 / 48.0));
+        const uint32_t k_lo = want_ksplit ? std::min(want_ksplit, nch) : 1, k_hi = want_ksplit ? k_lo : std::min(16u, nch);
+        for (uint32_t k = k_lo; k <= k_hi; ++k) {
+            SplitSchedule s;
+            const uint32_t per = (nch + k - 1) / k;
+            s.bn = bn;
+            s.ksplit = (nch + per - 1) / per;   // every slice holds at least one chunk
+            const int64_t pb = split_partial_bytes(M, N, s);
+            if (pb > partial_limit) continue;
+            const double waves = (double)((tiles * s.ksplit + pairs - 1) / pairs);
+            s.us = waves * (per * chunk + 5000 + 10.0 * bn) / 1900.0;
+            if (s.ksplit > 1) s.us += 3.0 + (double)pb / 2.0e6;   // written and read back, mostly in L2
+            if (!have || s.us < best.us * (1 - 1e-9)) { best = s; have = true; }
+        }
+    }
+    // more slices asked for than their partial sums may take: the most that fit
+    if (!have && want_ksplit > 1) return split_schedule(M, N, K, pairs, want_ksplit - 1, partial_limit);
+    return best;
+}
+
+}  // namespace comet

@@ -1,0 +1,54 @@
+"""The split GEMM's CTA-pair kernel at the edges of its tiles, chunks and K slices against the FP64
+oracle.  Bounds: two FP16 parts leave at most 2^-23 of an element's leading power of two and
+drop products below 2^-22, so with a few truncations per chunk and two levels of FP32 sums the
+normwise error of normal operands stays below 6e-7; rows far below the operand's largest
+element keep it relative to themselves down to 2^-16 (FP16's exponent range below 2^14)."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from helpers import empty_like_labels, from_dev, normwise, to_dev
+
+pytestmark = pytest.mark.gpu
+
+E = "C[m,n] = A[k,m] * B[k,n]"
+
+
+@pytest.fixture(scope="module")
+def comet():
+    import paper_2102_06827_gb300 as c
+    return c
+
+
+def run(comet, expr, ext, arrays, **kw):
+    import torch
+    p = comet.Plan(expr, ext, torch.float32, precision="split_bf16", **kw)
+    out = empty_like_labels([ext["m"], ext["n"]], torch.float32)
+    p.contract([to_dev(a, np.float32) for a in arrays], out, p.workspace())
+    comet.sync_status()
+    return from_dev(out).astype(np.float64)
+
+
+def f32(shape, seed, t, **kw):
+    return synth.tensor(shape, seed, t, **kw).astype(np.float32).astype(np.float64)
+
+
+@pytest.mark.parametrize("ksplit", [1, 2])
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (129, 49, 31), (257, 193, 65), (256, 192, 64), (255, 47, 129),
+                                   (513, 385, 200), (300, 200, 4096), (300, 200, 4097)])
+def test_tiles_chunks_and_slices(comet, M, N, K, ksplit):
+    ext = dict(m=M, n=N, k=K)
+    A, B = f32((K, M), 71, 0, kind="normal"), f32((K, N), 71, 1, kind="normal")
+    assert normwise(run(comet, E, ext, [A, B], ksplit=ksplit), oracle.einsum(E, A, B)) <= 6e-7
+    A, B = f32((K, M), 72, 0, kind="int", lo=-9, hi=9), f32((K, N), 72, 1, kind="int", lo=-9, hi=9)
+    assert np.array_equal(run(comet, E, ext, [A, B], ksplit=ksplit), oracle.einsum(E, A, B))
+
+
+def test_small_rows_keep_their_relative_precision(comet):
+    ext = dict(m=200, n=96, k=300)
+    A, B = f32((300, 200), 73, 0, kind="normal"), f32((300, 96), 73, 1, kind="normal")
+    A = A * 2.0 ** -(np.arange(200) % 17)       # rows from the largest element's size to 2^-16 of it
+    C, ref = run(comet, E, ext, [A, B]), oracle.einsum(E, A, B)
+    rows = np.abs(C - ref).max(axis=1) / np.abs(ref).max(axis=1)
+    assert rows.max() <= 1e-6
