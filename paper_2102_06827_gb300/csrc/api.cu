@@ -196,7 +196,7 @@ static comet_status_t run_plan(const Plan &P, const void *const *inputs, void *o
         const DbgRange rb = slot_range(P, st.b, inputs, output, ws);
         char *w = static_cast<char *>(ws);
         void *sc_a = w + st.ws_scales, *sc_b = w + st.ws_scales + 8;
-        const bool split_like = st.kernel == KK_GEMM_SPLIT || st.kernel == KK_GEMM_EMU;
+        const bool split_like = (st.kernel == KK_GEMM_SPLIT && !st.small) || st.kernel == KK_GEMM_EMU;
         if (split_like) {   // operand scales over the whole operands (every batch index shares them)
             const Slot &sa_ = P.slots[st.form.swap ? st.b : st.a], &sb_ = P.slots[st.form.swap ? st.a : st.b];
             const void *xa = st.form.swap ? pb : pa, *xb = st.form.swap ? pa : pb;
@@ -261,14 +261,17 @@ static comet_status_t run_plan(const Plan &P, const void *const *inputs, void *o
                 if (e != cudaSuccess) return cuda_status(e, "gemv kernel");
                 continue;
             }
-            if (st.kernel == KK_GEMM_F64) {
+            if (st.kernel == KK_GEMM_F64 || st.small) {
                 bool ak = g.k.n > 0 && (g.k.s0[0] == 1 || g.ma.n == 0 || (g.ma.s0[0] != 1 && g.k.s0[0] < g.ma.s0[0]));
                 bool bk = g.k.n > 0 && (g.k.s1[0] == 1 || g.nb.n == 0 || (g.nb.s0[0] != 1 && g.k.s1[0] < g.nb.s0[0]));
-                {
+                if (st.small) {
+                    ProfScope ps(PK_SPLIT, stream);
+                    e = launch_gemm_small(g, ak, bk, stream);
+                } else {
                     ProfScope ps(PK_F64, stream);
                     e = launch_gemm_f64(g, es, ak, bk, stream);
                 }
-                if (e != cudaSuccess) return cuda_status(e, "gemm_f64 kernel");
+                if (e != cudaSuccess) return cuda_status(e, st.small ? "small gemm kernel" : "gemm_f64 kernel");
                 continue;
             }
             XposeParams xa = st.pre_a, xb = st.pre_b;

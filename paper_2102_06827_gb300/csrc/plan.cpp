@@ -1073,6 +1073,17 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
                                                      st.want_ksplit, limit / 256 * 256);
             st.ksplit = sch.ksplit;
             st.tile_n = sch.bn;
+            // one launch on the FP32 pipes where that is modelled faster than the split form's chain
+            // (about 12 us of pre-passes and launches around its GEMM); asking for K slices or for the
+            // fault injection keeps the split form
+            const Slot &sm = P->slots[st.form.swap ? st.b : st.a], &sn = P->slots[st.form.swap ? st.a : st.b];
+            auto run = [&](const Slot &s, const std::vector<int> &rows) {
+                auto t = slot_strides(*P, s);
+                return std::max(contiguous_run(rows, t, P->extent), contiguous_run(st.form.K, t, P->extent));
+            };
+            const bool long_runs = run(sm, st.form.M) >= 16 && run(sn, st.form.N) >= 16;
+            st.small = P->dtype == COMET_F32 && opts.ksplit <= 0 && !(opts.debug_flags & 1) &&
+                       small_gemm_us((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, long_runs) < sch.us + 12.0;
             bk = (size_t)split_partial_bytes((uint64_t)rows_a, (uint64_t)rows_b, sch);
             const int64_t tiles = ((rows_a + 127) / 128) * ((rows_b + 255) / 256), tail = tiles % 152;
             st.tail_tiles = 0;
@@ -1274,7 +1285,7 @@ std::string describe_plan(const Plan &P) {
               << ",\"n_forms\":" << s.n_forms << ",\"form_index\":" << s.form_index
               << ",\"cost_s\":" << s.form.cost << ",\"pre_bytes\":" << s.form.pre_bytes
               << ",\"eff_store\":" << s.form.eff_store << ",\"flops\":" << s.flops
-              << ",\"ksplit\":" << s.ksplit << ",\"tile_n\":" << s.tile_n;
+              << ",\"ksplit\":" << s.ksplit << ",\"tile_n\":" << s.tile_n << ",\"small\":" << (s.small ? "true" : "false");
             if (s.kernel == KK_GEMM_SPLIT)
                 o << ",\"tail_tiles\":" << s.tail_tiles << ",\"tail_slices\":" << s.tail_slices;
         }

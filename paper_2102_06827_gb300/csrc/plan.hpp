@@ -73,6 +73,7 @@ struct Step {
     size_t ws_scales = 0;        // two 8-byte words: max |A|, max |B| of the step's operands
     int64_t kpad = 0;
     uint32_t want_ksplit = 0;    // split GEMM: the caller's K slices (0 = free)
+    bool small = false;          // split GEMM of FP32 operands: runs as one launch (k_gemm_small.cu)
     uint32_t ksplit = 1, tile_n = 0;   // split GEMM: K slices and tile width on 152 SMs (the launch
                                        // makes the same choice from the device's own count)
     size_t ws_ksplit = 0;        // workspace offset of the slices' FP32 partials

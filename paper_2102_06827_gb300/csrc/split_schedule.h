@@ -71,4 +71,13 @@ inline SplitSchedule split_schedule(uint64_t M, uint64_t N, uint64_t K, uint32_t
     return best;
 }
 
+// Modelled time of the same GEMM as one launch on the FP32 pipes (k_gemm_small.cu), at 1.9 GHz: tiles
+// of 16 x 16 over 152 SMs, 900 clocks a tile and 22 per K value, or 42 where an operand's contiguous
+// runs are short (its 4-byte gathers then take as many cache lines), and 3 us of launch.  Measured:
+// 192^3 6.1 us, 300^3 14.4, 1000 x 1000 x 16 18.5; with runs of 8 and 10 values 6.9, 26.4, -.
+inline double small_gemm_us(uint64_t M, uint64_t N, uint64_t K, bool long_runs) {
+    const uint64_t tiles = ((M + 15) / 16) * ((N + 15) / 16);
+    return 3.0 + (double)((tiles + 151) / 152) * (900.0 + (double)K * (long_runs ? 22.0 : 42.0)) / 1900.0;
+}
+
 }  // namespace comet
