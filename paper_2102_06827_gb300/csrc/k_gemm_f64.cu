@@ -7,7 +7,7 @@
 // Arithmetic: FP64 tensor-core MMA (mma.sync.m8n8k4 f64) with FP64 accumulation; FP32-stored
 // operands are widened exactly on load and the result is rounded once on store.
 //
-// Blocking: TM x TM output tile per CTA (TM = 64; 32 when 64-wide tiles would leave SMs idle),
+// Blocking: TM x TM output tile per CTA (TM = 64, 32 or 16, whichever loads the SMs most evenly),
 // K in blocks of 16, four warps of TM/2 x TM/2; the next K block is loaded into registers while
 // the current one is multiplied (double-buffered shared memory).
 #include <cuda_runtime.h>
@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(FTHREADS) gemm_f64_kernel(const GemmParams p) 
         }
 #pragma unroll
         for (int k4 = 0; k4 < FBK / 4; ++k4) {
+            if (kb * FBK + k4 * 4 >= p.K) break;   // no FP64 MMAs on a tail of zeros
             const int kk = k4 * 4 + (lane & 3);
             double af[FI], bf[FI];
 #pragma unroll
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(FTHREADS) gemm_f64_kernel(const GemmParams p) 
                 if (n0 + nl >= p.N) continue;
                 TIn *dst = C + c_row[ml] + c_col[nl];
                 if (!dbg_ok(p.dbg_c, dst, (int)sizeof(TIn), p.status)) continue;
-                double v = p.alpha * acc[i][j][h];
+                double v = p.alpha == 1.0 ? acc[i][j][h] : p.alpha * acc[i][j][h];   // the FP64 pipe is what is short
                 if (p.beta != 0.0) v += p.beta * (double)*dst;
                 *dst = (TIn)v;
             }
@@ -169,14 +170,24 @@ cudaError_t launch_gemm_f64(const GemmParams &p, int elem_bytes, bool a_kcontig,
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         return n;
     }();
-    // 64-wide tiles unless they would leave SMs idle
-    const uint64_t tiles64 = (uint64_t)((p.M + 63) / 64) * ((p.N + 63) / 64);
-    const int tm = tiles64 < (uint64_t)sms ? 32 : 64;
+    // The FP64 pipe (3.8 flops per clock and SM) hides everything else, so what counts is how evenly
+    // the tiles fall on the SMs, padding included: the tile edge with the fewest outputs on the busiest SM, the
+    // larger edge unless a smaller one saves 3 %.  Extents 24 (576 x 576, K = 24): 324 tiles of 32 are
+    // three on some SMs (33 us with K padded to 32), 1296 of 16 are nine at most.
+    int tm = 64;
+    double least = 0;
+    for (int edge : {64, 32, 16}) {
+        const uint64_t tiles = (uint64_t)((p.M + edge - 1) / edge) * ((p.N + edge - 1) / edge);
+        const double load = (double)((tiles + sms - 1) / sms) * edge * edge;
+        if ((p.N + edge - 1) / edge > 65535) continue;
+        if (edge == 64 || load < 0.97 * least) { tm = edge; least = load; }
+    }
     dim3 grid((p.M + tm - 1) / tm, (p.N + tm - 1) / tm);
     if (grid.y > 65535) return cudaErrorInvalidConfiguration;
 #define CM_LAUNCH(T, a, b)                                                               \
     do {                                                                                 \
-        if (tm == 32) gemm_f64_kernel<T, a, b, 32><<<grid, FTHREADS, 0, s>>>(p);         \
+        if (tm == 16) gemm_f64_kernel<T, a, b, 16><<<grid, FTHREADS, 0, s>>>(p);         \
+        else if (tm == 32) gemm_f64_kernel<T, a, b, 32><<<grid, FTHREADS, 0, s>>>(p);    \
         else gemm_f64_kernel<T, a, b, 64><<<grid, FTHREADS, 0, s>>>(p);                  \
     } while (0)
     if (elem_bytes == 8) {
