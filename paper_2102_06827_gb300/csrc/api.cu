@@ -138,10 +138,16 @@ static DbgRange slot_range(const Plan &P, int slot, const void *const *inputs, v
     return dbg_range(static_cast<char *>(ws) + s.ws_off, s.elems * es);
 }
 
-// max |x| over the elements of a step operand (a strided walk for views)
-static cudaError_t operand_absmax(const Slot &s, const void *p, int es, void *out, cudaStream_t stream) {
-    if (s.view) return launch_absmax_view(p, s.vradix, es, out, stream);
-    return launch_absmax(p, s.elems, es, out, stream);
+// abs-max argument of a step operand (a strided walk for views) with its slots
+static AbsmaxArg absmax_arg(const Slot &s, const void *p, int es, char *slots, uint32_t room) {
+    AbsmaxArg a;
+    a.x = p;
+    a.n = s.elems;
+    a.r = s.vradix;
+    a.view = s.view ? 1 : 0;
+    a.blocks = absmax_blocks(s.elems, es, room);
+    a.slots = slots;
+    return a;
 }
 
 static comet_status_t run_plan(const Plan &P, const void *const *inputs, void *output, void *ws,
@@ -197,22 +203,14 @@ static comet_status_t run_plan(const Plan &P, const void *const *inputs, void *o
         char *w = static_cast<char *>(ws);
         void *sc_a = w + st.ws_scales, *sc_b = w + st.ws_scales + 8;
         const bool split_like = (st.kernel == KK_GEMM_SPLIT && !st.small) || st.kernel == KK_GEMM_EMU;
+        AbsmaxArg arg_a, arg_b;
         if (split_like) {   // operand scales over the whole operands (every batch index shares them)
             const Slot &sa_ = P.slots[st.form.swap ? st.b : st.a], &sb_ = P.slots[st.form.swap ? st.a : st.b];
             const void *xa = st.form.swap ? pb : pa, *xb = st.form.swap ? pa : pb;
-            if (!sa_.view && !sb_.view) {   // both dense: one launch (sc_b is the word after sc_a)
-                ProfScope ps(PK_PREPASS, stream);
-                e = launch_absmax2(xa, sa_.elems, xb, sb_.elems, es, sc_a, stream);
-            } else {
-                {
-                    ProfScope ps(PK_PREPASS, stream);
-                    e = operand_absmax(sa_, xa, es, sc_a, stream);
-                }
-                if (e == cudaSuccess) {
-                    ProfScope ps(PK_PREPASS, stream);
-                    e = operand_absmax(sb_, xb, es, sc_b, stream);
-                }
-            }
+            arg_a = absmax_arg(sa_, xa, es, w + st.ws_slots, st.n_slots);
+            arg_b = absmax_arg(sb_, xb, es, w + st.ws_slots + 8 * st.n_slots, st.n_slots);
+            ProfScope ps(PK_PREPASS, stream);
+            e = launch_absmax(arg_a, arg_b, es, stream);
             if (e != cudaSuccess) return cuda_status(e, "split pre-pass (scales)");
         }
         // one pass of the step's kernels per batch index (a single pass without batch labels;
@@ -275,8 +273,10 @@ static comet_status_t run_plan(const Plan &P, const void *const *inputs, void *o
                 continue;
             }
             XposeParams xa = st.pre_a, xb = st.pre_b;
-            xa.in = g.A; xa.out = w + st.ws_parts_a; xa.scale_bits = sc_a;
-            xb.in = g.B; xb.out = w + st.ws_parts_b; xb.scale_bits = sc_b;
+            xa.in = g.A; xa.out = w + st.ws_parts_a; xa.scale_out = sc_a;
+            xb.in = g.B; xb.out = w + st.ws_parts_b; xb.scale_out = sc_b;
+            xa.slots = arg_a.slots; xa.n_slots = arg_a.blocks; xa.late_wait = 0;
+            xb.slots = arg_b.slots; xb.n_slots = arg_b.blocks; xb.late_wait = 1;
             const int64_t n_planes = st.kernel == KK_GEMM_EMU ? 6 : 2;
             xa.dbg_in = g.dbg_a; xa.dbg_out = dbg_range(xa.out, n_planes * xa.out_plane * 2);
             xb.dbg_in = g.dbg_b; xb.dbg_out = dbg_range(xb.out, n_planes * xb.out_plane * 2);
@@ -470,13 +470,22 @@ static comet_status_t run_host_pipe(const Plan &P, int n_calls, const void *cons
     auto prep = [&](cudaEvent_t ready, char *src, int64_t n_elems, void *scale, const XposeParams &tmpl,
                     int vec, int vout, char *planes, cudaEvent_t done) {
         cudaError_t ee = cudaStreamWaitEvent(s, ready, 0);
+        AbsmaxArg part;
         if (ee == cudaSuccess) {
             ProfScope ps(PK_PREPASS, s);
-            ee = launch_absmax(src, n_elems, (int)es, scale, s);
+            AbsmaxArg none;
+            none.blocks = 0;
+            part.x = src;
+            part.n = n_elems;
+            part.view = 0;
+            part.blocks = absmax_blocks(n_elems, (int)es, st.n_slots);
+            part.slots = w + st.ws_slots;
+            ee = launch_absmax(part, none, (int)es, s);
         }
         if (ee == cudaSuccess) {
             XposeParams xp = tmpl;
-            xp.in = src; xp.out = planes; xp.scale_bits = scale;
+            xp.in = src; xp.out = planes; xp.scale_out = scale;
+            xp.slots = part.slots; xp.n_slots = part.blocks; xp.late_wait = 0;
             xp.dbg_in = dbg_range(src, n_elems * (int64_t)es);
             xp.dbg_out = dbg_range(planes, (int64_t)n_planes * xp.out_plane * 2);
             xp.status = status;

@@ -109,6 +109,7 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
 
     auto fail = [&]() {
         *abort_flag = 1;
@@ -304,6 +305,7 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
             }
         }
     }
+    pdl_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -378,7 +380,7 @@ cudaError_t launch_gemm_emu(const GemmParams &p, const void *parts_a, const void
         cudaFuncSetAttribute(gemm_emu_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
         attr_set = true;
     }
-    gemm_emu_kernel<<<ctas, THREADS, SMEM_BYTES, s>>>(ta, tb, p, x);
+    launch_pdl(gemm_emu_kernel, ctas, THREADS, SMEM_BYTES, s, ta, tb, p, x);
     return cudaGetLastError();
 }
 

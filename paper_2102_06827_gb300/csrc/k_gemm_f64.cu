@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(FTHREADS) gemm_f64_kernel(const GemmParams p) 
         }
     };
     k_offsets(0, 0);
+    pdl_wait();
     __syncthreads();
 
     double acc[FI][FI][2];
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(FTHREADS) gemm_f64_kernel(const GemmParams p) 
         __syncthreads();
     }
 
+    pdl_launch();
     // epilogue: C[m,n] = alpha * acc (+ beta * C), stored through the C strides of M and N
     TIn *C = reinterpret_cast<TIn *>(p.C);
 #pragma unroll
@@ -186,9 +188,9 @@ cudaError_t launch_gemm_f64(const GemmParams &p, int elem_bytes, bool a_kcontig,
     if (grid.y > 65535) return cudaErrorInvalidConfiguration;
 #define CM_LAUNCH(T, a, b)                                                               \
     do {                                                                                 \
-        if (tm == 16) gemm_f64_kernel<T, a, b, 16><<<grid, FTHREADS, 0, s>>>(p);         \
-        else if (tm == 32) gemm_f64_kernel<T, a, b, 32><<<grid, FTHREADS, 0, s>>>(p);    \
-        else gemm_f64_kernel<T, a, b, 64><<<grid, FTHREADS, 0, s>>>(p);                  \
+        if (tm == 16) launch_pdl(gemm_f64_kernel<T, a, b, 16>, grid, FTHREADS, 0, s, p);         \
+        else if (tm == 32) launch_pdl(gemm_f64_kernel<T, a, b, 32>, grid, FTHREADS, 0, s, p);    \
+        else launch_pdl(gemm_f64_kernel<T, a, b, 64>, grid, FTHREADS, 0, s, p);                  \
     } while (0)
     if (elem_bytes == 8) {
         if (a_kcontig && b_kcontig) CM_LAUNCH(double, true, true);

@@ -1,7 +1,8 @@
 // Small FP32 contractions: one launch, no pre-pass, no scratch.
 //
 // A GEMM of a few million multiply-adds is over in a microsecond or two on the FP32 pipes, while the
-// split form needs its chain of launches (abs-max, two splits, tcgen05 GEMM) whatever the size.  So
+// split form needs its chain of launches (abs-max, two splits, tcgen05 GEMM) whatever the size: 11 us
+// at M = N = K = 192 (18 before those launches overlapped) against 5.5 here.  So
 // steps below the line that small_gemm_us / the split model draw run here: operands are gathered
 // through their own strides (the transposes of TTGT folded into the loads), products and sums are
 // FP32, and every addition's rounding error is kept in a second sum (the error of an FMA into s is
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(sg::T) gemm_small_kernel(const GemmParams p) {
         if (t - TM < cols) radix_offsets(p.nb, n0 + t - TM, o0, o1);
         b_col[t - TM] = o0; c_col[t - TM] = o1;
     }
+    pdl_wait();
     const float *A = reinterpret_cast<const float *>(p.A), *B = reinterpret_cast<const float *>(p.B);
     const int kq = t >> 6, q = t & 63, tm = (q & 7) * 2, tn = (q >> 3) * 2;   // 2 x 2 outputs, every fourth pair of k
     float s[2][2] = {}, c[2][2] = {};
@@ -127,6 +129,7 @@ __global__ void __launch_bounds__(sg::T) gemm_small_kernel(const GemmParams p) {
 #pragma unroll
         for (int j = 0; j < 2; ++j) part[(kq * TM + tn + j) * TM + tm + i] = make_float2(s[i][j], c[i][j]);
     __syncthreads();
+    pdl_launch();
     const int r = t & 15, n = t >> 4;
     if (r >= rows || n >= cols) return;
     float hi = 0.0f, lo = 0.0f;
@@ -164,10 +167,10 @@ cudaError_t launch_gemm_small(const GemmParams &p, bool a_kcontig, bool b_kconti
     if (p.M == 0 || p.N == 0) return cudaSuccess;
     const dim3 grid((p.M + TM - 1) / TM, (p.N + TM - 1) / TM);
     if (grid.y > 65535) return cudaErrorInvalidConfiguration;
-    if (a_kcontig && b_kcontig) gemm_small_kernel<true, true><<<grid, T, SMEM, s>>>(p);
-    else if (a_kcontig) gemm_small_kernel<true, false><<<grid, T, SMEM, s>>>(p);
-    else if (b_kcontig) gemm_small_kernel<false, true><<<grid, T, SMEM, s>>>(p);
-    else gemm_small_kernel<false, false><<<grid, T, SMEM, s>>>(p);
+    if (a_kcontig && b_kcontig) launch_pdl(gemm_small_kernel<true, true>, grid, T, SMEM, s, p);
+    else if (a_kcontig) launch_pdl(gemm_small_kernel<true, false>, grid, T, SMEM, s, p);
+    else if (b_kcontig) launch_pdl(gemm_small_kernel<false, true>, grid, T, SMEM, s, p);
+    else launch_pdl(gemm_small_kernel<false, false>, grid, T, SMEM, s, p);
     return cudaGetLastError();
 }
 

@@ -181,6 +181,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
     cluster_sync();   // both CTAs' barriers are set up before either CTA signals the other
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();       // the pre-passes' planes and scales, and whoever read or wrote C before
 
     auto fail = [&]() {
         *abort_flag = 1;
@@ -261,7 +262,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
         const uint32_t gn = x.bn / 3, g0 = (uint32_t)((warp - 4) >> 2) * gn;   // columns g0 .. g0 + gn - 1
         const int et = threadIdx.x - 128;           // 0..383
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
-        const int e_sum = scale_exponent<TOut>(x.scale_a) + scale_exponent<TOut>(x.scale_b);
+        const int e_sum = half_exponent<TOut>(scale_exponent<TOut>(x.scale_a)) +
+                          half_exponent<TOut>(scale_exponent<TOut>(x.scale_b));
         // 2^(eA+eB-28) in two factors: the sums carry 2^28 more than the result's scale
         constexpr float kShift = 1.0f / (float)(1 << (2 * kHalfShift));
         const uint32_t tempty0 = map_to_rank(tempty, 0);
@@ -360,6 +362,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
             }
         }
     }
+    pdl_launch();
     tc_fence_before();
     __syncthreads();
     cluster_sync();   // neither CTA frees its tensor memory or leaves while the other may still use it
@@ -388,6 +391,7 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmParams p, c
     }
     int64_t r0 = 0, c_row = 0;
     if (m < p.M) radix_offsets(p.ma, m, r0, c_row);
+    pdl_wait();
     __syncthreads();
     if (m >= p.M) return;
     const size_t slice = (size_t)x.m_tiles * x.n_tiles * 2 * x.bn * BM;
@@ -468,7 +472,7 @@ static void launch_split_kernel(const CUtensorMap &ta, const CUtensorMap &tb, co
         return true;
     }();
     (void)attr;
-    gemm_split_kernel<TOut, KSPLIT><<<ctas, split::THREADS, split::SMEM_BYTES, s>>>(ta, tb, p, x);
+    launch_pdl(gemm_split_kernel<TOut, KSPLIT>, ctas, split::THREADS, split::SMEM_BYTES, s, ta, tb, p, x);
 }
 
 cudaError_t launch_gemm_split(const GemmParams &p, const void *parts_a, const void *parts_b,
@@ -507,8 +511,8 @@ cudaError_t launch_gemm_split(const GemmParams &p, const void *parts_a, const vo
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || x.ksplit == 1) return e;
     const uint32_t blocks = x.m_tiles * x.n_tiles * 2 * (x.bn / STRIP);
-    if (out_bytes == 8) split_reduce_kernel<double><<<blocks, 256, 0, s>>>(p, x);
-    else split_reduce_kernel<float><<<blocks, 256, 0, s>>>(p, x);
+    if (out_bytes == 8) launch_pdl(split_reduce_kernel<double>, blocks, 256, 0, s, p, x);
+    else launch_pdl(split_reduce_kernel<float>, blocks, 256, 0, s, p, x);
     return cudaGetLastError();
 }
 

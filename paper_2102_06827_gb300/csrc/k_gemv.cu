@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(gv::T) gemv_partial_kernel(const GemvParams p)
     const uint32_t nk = min((uint32_t)KC, p.K - k0), nn = min((uint32_t)NT, p.N - n0);
     int64_t bo_v = 0, bo_x = 0;
     radix_offsets(p.bv, bi, bo_v, bo_x);
+    pdl_wait();
     const T *v = reinterpret_cast<const T *>(p.v) + bo_v;
     const T *X = reinterpret_cast<const T *>(p.X) + bo_x;
     for (uint32_t i = t; i < (uint32_t)KC; i += gv::T) {
@@ -79,6 +80,7 @@ __global__ void __launch_bounds__(gv::T) gemv_partial_kernel(const GemvParams p)
         n_off[i] = ox;
     }
     __syncthreads();
+    pdl_launch();   // (a block's own loads are still to come: the next kernel is the small finish)
     double *out = p.partial + ((size_t)bi * p.nchunks + blockIdx.y) * p.N;
     if (NFAST) {
         // threads along n (contiguous in X), two k phases
@@ -115,6 +117,8 @@ __global__ void __launch_bounds__(gv::T) gemv_partial_kernel(const GemvParams p)
 
 template <typename T>
 __global__ void __launch_bounds__(256) gemv_finish_kernel(const GemvParams p) {
+    pdl_wait();
+    pdl_launch();
     const uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= (uint64_t)p.n_batch * p.N) return;
     const uint32_t bi = (uint32_t)(i / p.N), n = (uint32_t)(i - (uint64_t)bi * p.N);
@@ -140,13 +144,13 @@ cudaError_t launch_gemv(const GemvParams &p, int elem_bytes, cudaStream_t s) {
     const dim3 grid1((uint32_t)(tiles * p.n_batch), p.nchunks);
     const uint32_t grid2 = (uint32_t)(((uint64_t)p.n_batch * p.N + 255) / 256);
     if (elem_bytes == 4) {
-        if (p.n_fast) gemv_partial_kernel<float, true><<<grid1, gv::T, 0, s>>>(p);
-        else gemv_partial_kernel<float, false><<<grid1, gv::T, 0, s>>>(p);
-        gemv_finish_kernel<float><<<grid2, 256, 0, s>>>(p);
+        if (p.n_fast) launch_pdl(gemv_partial_kernel<float, true>, grid1, gv::T, 0, s, p);
+        else launch_pdl(gemv_partial_kernel<float, false>, grid1, gv::T, 0, s, p);
+        launch_pdl(gemv_finish_kernel<float>, grid2, 256, 0, s, p);
     } else {
-        if (p.n_fast) gemv_partial_kernel<double, true><<<grid1, gv::T, 0, s>>>(p);
-        else gemv_partial_kernel<double, false><<<grid1, gv::T, 0, s>>>(p);
-        gemv_finish_kernel<double><<<grid2, 256, 0, s>>>(p);
+        if (p.n_fast) launch_pdl(gemv_partial_kernel<double, true>, grid1, gv::T, 0, s, p);
+        else launch_pdl(gemv_partial_kernel<double, false>, grid1, gv::T, 0, s, p);
+        launch_pdl(gemv_finish_kernel<double>, grid2, 256, 0, s, p);
     }
     return cudaGetLastError();
 }

@@ -32,16 +32,43 @@ struct alignas(sizeof(T) * N) Vec {
     T v[N];
 };
 
-// scale of a pre-pass: the operand's exponent (OP_SPLIT6) and 2^(14-e) as two factors (OP_SPLIT)
+// scale of a pre-pass: the operand's exponent (OP_SPLIT6) or its factor (OP_SPLIT), from the
+// maximum over the slots of its abs-max
 template <int OP, typename T>
 struct OpScale {
+    static constexpr bool kScaled = OP == OP_SPLIT || OP == OP_SPLIT6;
     int e = 0;
-    T s0 = 1, s1 = 1;
-    __device__ __forceinline__ explicit OpScale(const XposeParams &p) {
-        if constexpr (OP == OP_SPLIT || OP == OP_SPLIT6) e = scale_exponent<T>(p.scale_bits);
-        if constexpr (OP == OP_SPLIT) half_scales<T>(e, s0, s1);
+    HalfScale<T> half;
+    __device__ __forceinline__ OpScale() {}
+    __device__ __forceinline__ explicit OpScale(T largest) {
+        if constexpr (kScaled) e = exponent_of<T>(largest);
+        if constexpr (OP == OP_SPLIT) half = HalfScale<T>(half_exponent<T>(e));
+    }
+    __device__ __forceinline__ static T largest(const XposeParams &p) {
+        if constexpr (kScaled) {
+            const T m = slots_max<T>(p.slots, p.n_slots);
+            // the grid's first thread keeps the maximum for the GEMM
+            if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<T *>(p.scale_out) = m;
+            return m;
+        }
+        return 0;
     }
 };
+
+// Start of a kernel's memory work: the kernel before this one has ended.  A pre-pass that follows
+// the other operand's (late_wait) reads and writes nothing of that kernel's and starts at once:
+// that one let it begin only after its own wait, so everything earlier has ended.
+template <int OP>
+__device__ __forceinline__ void xpose_begin(const XposeParams &p) {
+    if (!((OP == OP_SPLIT || OP == OP_SPLIT6) && p.late_wait)) pdl_wait();
+    if (OP == OP_SPLIT || OP == OP_SPLIT6) pdl_launch();
+}
+
+template <int OP>
+__device__ __forceinline__ void xpose_end(const XposeParams &p) {
+    if ((OP == OP_SPLIT || OP == OP_SPLIT6) && p.late_wait) pdl_wait();
+    if (!(OP == OP_SPLIT || OP == OP_SPLIT6)) pdl_launch();
+}
 
 template <int OP, typename T, int VO>
 __device__ __forceinline__ void emit(const XposeParams &p, int64_t off, const T (&x)[VO], const OpScale<OP, T> &e) {
@@ -71,7 +98,7 @@ __device__ __forceinline__ void emit(const XposeParams &p, int64_t off, const T 
     } else if constexpr (OP == OP_SPLIT) {
         Vec<VO, __half> h, l;
 #pragma unroll
-        for (int q = 0; q < VO; ++q) split2<T>(x[q], e.s0, e.s1, h.v[q], l.v[q]);
+        for (int q = 0; q < VO; ++q) e.half.split(x[q], h.v[q], l.v[q]);
         __half *o = reinterpret_cast<__half *>(p.out) + off;
         if (!dbg_ok(p.dbg_out, o, 2 * (p.out_plane + VO), p.status)) return;   // both planes
         *reinterpret_cast<Vec<VO, __half> *>(o) = h;
@@ -154,8 +181,9 @@ __global__ void __launch_bounds__(XT, 8) xpose_tile_kernel(const XposeParams p) 
         ro.s = (int32_t)(w * nv * pitch + u);
         out_row[r] = ro;
     }
+    xpose_begin<OP>(p);
     __syncthreads();
-    const OpScale<OP, T> e(p);
+    __shared__ T largest;
     {   // loads: p.ll threads per row, each with a fixed u; batches of rows in flight together
         const uint32_t lanes = p.ll, rpp = p.rpp_l;
         const uint32_t r0 = fd_div(t, p.fd_ll);
@@ -174,6 +202,11 @@ __global__ void __launch_bounds__(XT, 8) xpose_tile_kernel(const XposeParams p) 
                     else
                         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src + in_row[row]) : "memory");
                 }
+            }
+            // the first warp looks the scale up while the copies are in flight
+            if (OpScale<OP, T>::kScaled && t < 32) {
+                const T m = OpScale<OP, T>::largest(p);
+                if (t == 0) largest = m;
             }
             asm volatile("cp.async.wait_all;\n" ::: "memory");
         } else if (r0 < rpp && u < nu) {
@@ -202,7 +235,12 @@ __global__ void __launch_bounds__(XT, 8) xpose_tile_kernel(const XposeParams p) 
             }
         }
     }
+    if (VI != 1 && OpScale<OP, T>::kScaled && t < 32) {
+        const T m = OpScale<OP, T>::largest(p);
+        if (t == 0) largest = m;
+    }
     __syncthreads();
+    const OpScale<OP, T> e(OpScale<OP, T>::kScaled ? largest : T(0));
     {   // stores: p.sl threads per row, each with a fixed v
         const uint32_t lanes = p.sl, rpp = p.rpp_s;
         const uint32_t r0 = fd_div(t, p.fd_sl);
@@ -221,6 +259,7 @@ __global__ void __launch_bounds__(XT, 8) xpose_tile_kernel(const XposeParams p) 
             }
         }
     }
+    xpose_end<OP>(p);
 }
 
 // Copy mode: input and output share the stride-1 dim U (a single digit, affine on both sides
@@ -241,15 +280,19 @@ __global__ void __launch_bounds__(XT, 6) xpose_copy_kernel(const XposeParams p) 
         row_in[i] = (OFF)(a + (int64_t)u0 * su);
         row_out[i] = (OFF)(c + (int64_t)u0 * so);
     }
+    xpose_begin<OP>(p);
     __syncthreads();
     const T *__restrict__ in = reinterpret_cast<const T *>(p.in);
-    const OpScale<OP, T> e(p);
+    const OpScale<OP, T> e(OpScale<OP, T>::largest(p));
     constexpr int UB = VW * sizeof(T) >= 16 ? 4 : 8;
     const uint32_t lanes = p.ll;
     const uint32_t rpp = p.rpp_l;
     const uint32_t r0 = fd_div(t, p.fd_ll);
     const uint32_t u = (t - r0 * lanes) * VW;
-    if (!(r0 < rpp && u < nu)) return;
+    if (!(r0 < rpp && u < nu)) {
+        xpose_end<OP>(p);
+        return;
+    }
     const T *__restrict__ src = in + (int64_t)u * su;
     const int64_t uo = (int64_t)u * so;
     if constexpr (VW * sizeof(T) <= 8) {
@@ -304,6 +347,7 @@ __global__ void __launch_bounds__(XT, 6) xpose_copy_kernel(const XposeParams p) 
             }
         }
     }
+    xpose_end<OP>(p);
 }
 
 // A single long run (copy mode, R empty), cut into pieces of up to kXposeTile elements: every
@@ -316,7 +360,8 @@ __global__ void __launch_bounds__(XT) xpose_run_kernel(const XposeParams p) {
     const uint32_t nu = min(tu, p.u.total - u0);
     const int64_t su = p.u.s0[0], so = p.u.s1[0];
     const T *__restrict__ in = reinterpret_cast<const T *>(p.in);
-    const OpScale<OP, T> e(p);
+    xpose_begin<OP>(p);
+    const OpScale<OP, T> e(OpScale<OP, T>::largest(p));
     constexpr int UB = VW * sizeof(T) >= 16 ? 4 : 8;
     const int64_t ri = (int64_t)u0 * su, ro = (int64_t)u0 * so;
     const uint32_t nvec = nu / VW * VW;
@@ -341,10 +386,12 @@ __global__ void __launch_bounds__(XT) xpose_run_kernel(const XposeParams p) {
     }
     if (t < (int)(nu - nvec)) {
         const uint32_t u = nvec + t;
-        if (!dbg_ok(p.dbg_in, in + ri + (int64_t)u * su, (int)sizeof(T), p.status)) return;
-        T xs[1] = {in[ri + (int64_t)u * su]};
-        emit<OP, T, 1>(p, ro + (int64_t)u * so, xs, e);
+        if (dbg_ok(p.dbg_in, in + ri + (int64_t)u * su, (int)sizeof(T), p.status)) {
+            T xs[1] = {in[ri + (int64_t)u * su]};
+            emit<OP, T, 1>(p, ro + (int64_t)u * so, xs, e);
+        }
     }
+    xpose_end<OP>(p);
 }
 
 // every element of a dense buffer set to one value: grid-stride 16-byte stores, element tail
@@ -368,99 +415,78 @@ cudaError_t launch_fill(void *out, int64_t n, double value, int elem_bytes, cuda
     return cudaGetLastError();
 }
 
-// max |x| over a dense operand: grid-stride 16-byte loads, warp reduction, one atomic per warp
-// on the bit pattern (for non-negative IEEE values the bit order is the numeric order).  `bid`
-// and `nb` are this block's index and the block count among the blocks given to the operand.
+// The largest finite |x| of one or two operands.  Each block walks its share with four 16-byte loads
+// in flight per thread (a view: element by element through its radix, smallest stride first) and
+// writes the bits of its maximum into its own slot; the pre-passes take the maximum over the slots.
+// Bits, not values: for non-negative IEEE values their order is the numeric order, which keeps FP64
+// operands off the FP64 pipe.  Slots, not one word and atomics: nothing has to be cleared first, and
+// 20 thousand atomics on two words took 13 of 18 us on two operands of 11 MB.
+constexpr int AT = 1024;
+
 template <typename T>
-__device__ __forceinline__ void absmax_body(const T *__restrict__ x, int64_t n, int64_t bid, int64_t nb,
-                                            void *out_bits) {
-    constexpr int W = 16 / sizeof(T);
+__device__ __forceinline__ void absmax_part(const AbsmaxArg &a, uint32_t bid) {
     using U = typename std::conditional<sizeof(T) == 4, unsigned int, unsigned long long>::type;
-    T m = 0;
-    const int64_t nv = n / W;
-    const int64_t stride = nb * blockDim.x;
-    for (int64_t i = bid * (int64_t)blockDim.x + threadIdx.x; i < nv; i += stride) {
-        Vec<W, T> w = reinterpret_cast<const Vec<W, T> *>(x)[i];
+    constexpr U kSign = (U)1 << (8 * sizeof(U) - 1);
+    constexpr U kInf = sizeof(T) == 4 ? (U)0x7F800000u : (U)0x7FF0000000000000ull;
+    __shared__ U part[AT / 32];
+    U m = 0;
+    auto take = [&](U bits) {
+        bits &= ~kSign;
+        m = bits < kInf ? max(m, bits) : m;
+    };
+    const U *x = reinterpret_cast<const U *>(a.x);
+    const int64_t first = bid * (int64_t)AT + threadIdx.x, stride = a.blocks * (int64_t)AT;
+    if (!a.view) {
+        constexpr int W = 16 / sizeof(T), UB = 4;
+        const int64_t nv = a.n / W;
+        for (int64_t i = first; i < nv; i += UB * stride) {
+            Vec<W, U> w[UB];
 #pragma unroll
-        for (int q = 0; q < W; ++q) m = fmax(m, fabs(w.v[q]));
+            for (int j = 0; j < UB; ++j)
+                if (i + j * stride < nv) w[j] = reinterpret_cast<const Vec<W, U> *>(x)[i + j * stride];
+#pragma unroll
+            for (int j = 0; j < UB; ++j)
+                if (i + j * stride < nv) {
+#pragma unroll
+                    for (int q = 0; q < W; ++q) take(w[j].v[q]);
+                }
+        }
+        for (int64_t i = nv * W + first; i < a.n; i += stride) take(x[i]);
+    } else {
+        for (int64_t i = first; i < (int64_t)a.r.total; i += stride) {
+            int64_t o0 = 0, o1 = 0;
+            radix_offsets(a.r, (uint32_t)i, o0, o1);
+            take(x[o0]);
+        }
     }
-    for (int64_t i = nv * W + bid * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride)
-        m = fmax(m, fabs(x[i]));
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0) {
-        U bits;
-        memcpy(&bits, &m, sizeof(U));
-        atomicMax(reinterpret_cast<U *>(out_bits), bits);
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+    pdl_launch();
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        m = part[threadIdx.x];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (threadIdx.x == 0) *reinterpret_cast<U *>(static_cast<char *>(a.slots) + 8 * bid) = m;
     }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) absmax_kernel(const T *__restrict__ x, int64_t n, void *out_bits) {
-    absmax_body(x, n, blockIdx.x, gridDim.x, out_bits);
+__global__ void __launch_bounds__(AT) absmax_kernel(const __grid_constant__ AbsmaxArg a, const __grid_constant__ AbsmaxArg b) {
+    pdl_wait();
+    if (blockIdx.x < a.blocks) absmax_part<T>(a, blockIdx.x);
+    else absmax_part<T>(b, blockIdx.x - a.blocks);
 }
 
-// both operands of a split step in one launch: blocks [0, blocks0) take x0 (word 0 of out_bits),
-// the rest x1 (word 1, 8 bytes further)
-template <typename T>
-__global__ void __launch_bounds__(256) absmax2_kernel(const T *__restrict__ x0, int64_t n0, const T *__restrict__ x1,
-                                                      int64_t n1, int blocks0, void *out_bits) {
-    if ((int)blockIdx.x < blocks0) absmax_body(x0, n0, blockIdx.x, blocks0, out_bits);
-    else absmax_body(x1, n1, blockIdx.x - blocks0, gridDim.x - blocks0, static_cast<char *>(out_bits) + 8);
+uint32_t absmax_blocks(int64_t n, int elem_bytes, uint32_t room) {
+    const int64_t per = AT * 16 / elem_bytes;   // one 16-byte load per thread
+    return (uint32_t)std::max<int64_t>(1, std::min<int64_t>({(int64_t)room, 152, (n + per - 1) / per}));
 }
 
-static int absmax_blocks(int64_t n) { return (int)std::min<int64_t>(152 * 8, (n + 256 * 4 - 1) / (256 * 4)); }
-
-cudaError_t launch_absmax(const void *x, int64_t n, int elem_bytes, void *out_bits, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(out_bits, 0, 8, s);
-    if (e != cudaSuccess || n == 0) return e;
-    const int blocks = absmax_blocks(n);
-    if (elem_bytes == 4) absmax_kernel<float><<<blocks, 256, 0, s>>>(reinterpret_cast<const float *>(x), n, out_bits);
-    else absmax_kernel<double><<<blocks, 256, 0, s>>>(reinterpret_cast<const double *>(x), n, out_bits);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_absmax2(const void *x0, int64_t n0, const void *x1, int64_t n1, int elem_bytes, void *out_bits,
-                           cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(out_bits, 0, 16, s);
-    const int b0 = absmax_blocks(n0), b1 = absmax_blocks(n1);
-    if (e != cudaSuccess || b0 + b1 == 0) return e;
-    if (elem_bytes == 4)
-        absmax2_kernel<float><<<b0 + b1, 256, 0, s>>>(reinterpret_cast<const float *>(x0), n0,
-                                                      reinterpret_cast<const float *>(x1), n1, b0, out_bits);
-    else
-        absmax2_kernel<double><<<b0 + b1, 256, 0, s>>>(reinterpret_cast<const double *>(x0), n0,
-                                                       reinterpret_cast<const double *>(x1), n1, b0, out_bits);
-    return cudaGetLastError();
-}
-
-// max |x| over a strided view: each thread walks elements through the radix (smallest stride
-// first, so neighbouring threads touch neighbouring addresses where the view allows)
-template <typename T>
-__global__ void __launch_bounds__(256) absmax_view_kernel(const T *__restrict__ x, const Radix r, void *out_bits) {
-    using U = typename std::conditional<sizeof(T) == 4, unsigned int, unsigned long long>::type;
-    T m = 0;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < r.total; i += gridDim.x * blockDim.x) {
-        int64_t o0 = 0, o1 = 0;
-        radix_offsets(r, i, o0, o1);
-        m = fmax(m, fabs(x[o0]));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0) {
-        U bits;
-        memcpy(&bits, &m, sizeof(U));
-        atomicMax(reinterpret_cast<U *>(out_bits), bits);
-    }
-}
-
-cudaError_t launch_absmax_view(const void *x, const Radix &r, int elem_bytes, void *out_bits, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(out_bits, 0, 8, s);
-    if (e != cudaSuccess || r.total == 0) return e;
-    int blocks = (int)std::min<int64_t>(152 * 8, ((int64_t)r.total + 255) / 256);
-    if (elem_bytes == 4) absmax_view_kernel<float><<<blocks, 256, 0, s>>>(reinterpret_cast<const float *>(x), r, out_bits);
-    else absmax_view_kernel<double><<<blocks, 256, 0, s>>>(reinterpret_cast<const double *>(x), r, out_bits);
-    return cudaGetLastError();
+cudaError_t launch_absmax(const AbsmaxArg &a, const AbsmaxArg &b, int elem_bytes, cudaStream_t s) {
+    if (elem_bytes == 4) return launch_pdl(absmax_kernel<float>, a.blocks + b.blocks, AT, 0, s, a, b);
+    return launch_pdl(absmax_kernel<double>, a.blocks + b.blocks, AT, 0, s, a, b);
 }
 
 static uint32_t xpose_grid(const XposeParams &p) {
@@ -475,7 +501,7 @@ static void launch_tile(const XposeParams &p, uint32_t g, size_t smem, cudaStrea
         return true;
     }();
     (void)attr;
-    xpose_tile_kernel<OP, T, VI, VO, OFF><<<g, XT, smem, s>>>(p);
+    launch_pdl(xpose_tile_kernel<OP, T, VI, VO, OFF>, g, XT, smem, s, p);
 }
 
 // vector widths W (16 bytes), 2 (8 bytes, FP32 only) and 1, chosen at run time
@@ -503,20 +529,20 @@ static cudaError_t launch_op(const XposeParams &p, int vi, int vo, cudaStream_t 
     if (vo < 0) {   // copy mode
         const bool wide = -vo >= W && vi >= W;
         if (p.single_run) {
-            if (wide) xpose_run_kernel<OP, T, W><<<g, XT, 0, s>>>(p);
-            else xpose_run_kernel<OP, T, 1><<<g, XT, 0, s>>>(p);
+            if (wide) launch_pdl(xpose_run_kernel<OP, T, W>, g, XT, 0, s, p);
+            else launch_pdl(xpose_run_kernel<OP, T, 1>, g, XT, 0, s, p);
             return cudaGetLastError();
         }
         const size_t stage = (size_t)p.tu * p.tw * sizeof(T);   // asynchronous rows stage in shared memory
         const bool half = W == 4 && -vo >= 2 && vi >= 2;        // FP32 rows in 8-byte pieces
         if (p.off32) {
-            if (wide) xpose_copy_kernel<OP, T, W, int32_t><<<g, XT, 0, s>>>(p);
-            else if (half) xpose_copy_kernel<OP, T, (W == 4 ? 2 : 1), int32_t><<<g, XT, stage, s>>>(p);
-            else xpose_copy_kernel<OP, T, 1, int32_t><<<g, XT, stage, s>>>(p);
+            if (wide) launch_pdl(xpose_copy_kernel<OP, T, W, int32_t>, g, XT, 0, s, p);
+            else if (half) launch_pdl(xpose_copy_kernel<OP, T, (W == 4 ? 2 : 1), int32_t>, g, XT, stage, s, p);
+            else launch_pdl(xpose_copy_kernel<OP, T, 1, int32_t>, g, XT, stage, s, p);
         } else {
-            if (wide) xpose_copy_kernel<OP, T, W, int64_t><<<g, XT, 0, s>>>(p);
-            else if (half) xpose_copy_kernel<OP, T, (W == 4 ? 2 : 1), int64_t><<<g, XT, stage, s>>>(p);
-            else xpose_copy_kernel<OP, T, 1, int64_t><<<g, XT, stage, s>>>(p);
+            if (wide) launch_pdl(xpose_copy_kernel<OP, T, W, int64_t>, g, XT, 0, s, p);
+            else if (half) launch_pdl(xpose_copy_kernel<OP, T, (W == 4 ? 2 : 1), int64_t>, g, XT, stage, s, p);
+            else launch_pdl(xpose_copy_kernel<OP, T, 1, int64_t>, g, XT, stage, s, p);
         }
         return cudaGetLastError();
     }

@@ -98,7 +98,12 @@ struct XposeParams {
     const void *in;
     void *out;
     int64_t out_plane;             // split pre-pass: element distance between the 3 planes
-    const void *scale_bits;        // split pre-pass: device word holding the bits of max |x|
+    const void *slots;             // split pre-pass: n_slots 8-byte words, the bits of max |x| of a
+    uint32_t n_slots;              // part of the operand each
+    void *scale_out;               // split pre-pass: word that receives the bits of their maximum
+    int late_wait;                 // split pre-pass: the kernel before this one is the other operand's
+                                   // pre-pass; wait for its end before this kernel's own, not before
+                                   // the loads
     double alpha;                  // scaled copy: out = alpha * in (+ beta * out)
     double beta;
     uint32_t tu, tv, tw;           // tile extents along U, V and R (tu*tv*tw <= kXposeTile)

@@ -1050,6 +1050,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
     for (auto &s : P->slots)
         if (s.kind == SLOT_INTER) { s.ws_off = off; off = align(off + (size_t)s.elems * es); }
     size_t parts_base = off, parts_max = 0;
+    constexpr int64_t kSlots = 152;   // abs-max slots per operand (8 bytes each)
     for (auto &st : P->steps) {
         if (st.kernel != KK_GEMM_SPLIT && st.kernel != KK_GEMM_EMU) continue;
         int64_t Kx = prod_ext(P->extent, st.form.K);
@@ -1065,7 +1066,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             // static scratch when the plan without them would (three planes per operand were
             // kept before; the step's room is never less than theirs), else within 256 MB
             least = align((size_t)6 * rows_a * st.kpad) + align((size_t)6 * rows_b * st.kpad);
-            const int64_t fixed = COMET_NOALLOC_MAX_BYTES - 256;
+            const int64_t fixed = COMET_NOALLOC_MAX_BYTES - 256 - 16 * kSlots;
             const int64_t limit = (int64_t)(parts_base + least) <= fixed ? fixed - (int64_t)(parts_base + ba + bb)
                                                                          : (int64_t)256 << 20;
             st.want_ksplit = opts.ksplit > 0 ? (uint32_t)opts.ksplit : 0;
@@ -1074,7 +1075,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             st.ksplit = sch.ksplit;
             st.tile_n = sch.bn;
             // one launch on the FP32 pipes where that is modelled faster than the split form's chain
-            // (about 12 us of pre-passes and launches around its GEMM); asking for K slices or for the
+            // (about 9 us of pre-passes and launches around its GEMM); asking for K slices or for the
             // fault injection keeps the split form
             const Slot &sm = P->slots[st.form.swap ? st.b : st.a], &sn = P->slots[st.form.swap ? st.a : st.b];
             auto run = [&](const Slot &s, const std::vector<int> &rows) {
@@ -1083,7 +1084,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             };
             const bool long_runs = run(sm, st.form.M) >= 16 && run(sn, st.form.N) >= 16;
             st.small = P->dtype == COMET_F32 && opts.ksplit <= 0 && !(opts.debug_flags & 1) &&
-                       small_gemm_us((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, long_runs) < sch.us + 12.0;
+                       small_gemm_us((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, long_runs) < sch.us + 9.0;
             bk = (size_t)split_partial_bytes((uint64_t)rows_a, (uint64_t)rows_b, sch);
             const int64_t tiles = ((rows_a + 127) / 128) * ((rows_b + 255) / 256), tail = tiles % 152;
             st.tail_tiles = 0;
@@ -1138,8 +1139,18 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
     }
     bool any_split = false;
     for (auto &st : P->steps) any_split |= st.kernel == KK_GEMM_SPLIT || st.kernel == KK_GEMM_EMU;
-    for (auto &st : P->steps) st.ws_scales = parts_base + parts_max;
-    P->workspace = parts_base + parts_max + (any_split ? 256 : 0);
+    // after the parts: 256 bytes of scale words (slices of the host pipeline have one each) and the
+    // slots of the abs-max pass, one per block and operand; where those would put the plan past
+    // the library's static scratch, the 14 per operand that the scale words leave room for (a
+    // host-pipelined plan is larger than that scratch or its slices few)
+    const size_t scales_end = parts_base + parts_max + 256;
+    const bool room = scales_end > COMET_NOALLOC_MAX_BYTES || scales_end + 16 * kSlots <= COMET_NOALLOC_MAX_BYTES;
+    for (auto &st : P->steps) {
+        st.ws_scales = parts_base + parts_max;
+        st.ws_slots = room ? scales_end : st.ws_scales + 16;
+        st.n_slots = room ? kSlots : 14;
+    }
+    P->workspace = any_split ? scales_end + (room ? 16 * kSlots : 0) : parts_base + parts_max;
 
     // ---- precomputed parameter blocks ----
     for (auto &st : P->steps) {

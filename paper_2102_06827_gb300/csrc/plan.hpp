@@ -71,6 +71,8 @@ struct Step {
     // split path workspace for the parts: [2][rows][kpad] FP16 (split) or [6][rows][kpad] bf16 (emulated)
     size_t ws_parts_a = 0, ws_parts_b = 0;
     size_t ws_scales = 0;        // two 8-byte words: max |A|, max |B| of the step's operands
+    size_t ws_slots = 0;         // abs-max slots of A, then of B: n_slots 8-byte words each
+    uint32_t n_slots = 0;
     int64_t kpad = 0;
     uint32_t want_ksplit = 0;    // split GEMM: the caller's K slices (0 = free)
     bool small = false;          // split GEMM of FP32 operands: runs as one launch (k_gemm_small.cu)

@@ -3,6 +3,9 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
+#include <string.h>
+
+#include <type_traits>
 
 namespace comet {
 
@@ -43,22 +46,36 @@ __device__ __forceinline__ void split3(T x, int e, __nv_bfloat16 &h, __nv_bfloat
 // magnitude into [2^14, 2^15), so that the exponent range of FP16 lies below it).  The residual
 // x' - h is exact in the input precision and at most half a unit of h; what remains after l is at
 // most 2^-23 of the power of two below |x'| (never more than split3 leaves), or 2^-25 where l is
-// subnormal.  `s0`, `s1`: 2^(14-e) as a product of two powers of two, each inside the type's range.
+// subnormal.  FP32: e is at least -112, which keeps the factor a normal number (all of an operand
+// below 2^-112 is a multiple of 2^-149, so of 2^-23 once scaled: nothing is lost).  FP64: the
+// factor is a product of two, each inside the type's range.
 constexpr int kHalfShift = 14;
 
+// e of the split, from the exponent of the operand's largest magnitude
 template <typename T>
-__device__ __forceinline__ void half_scales(int e, T &s0, T &s1) {
-    const int s = kHalfShift - e, a = s / 2;
-    if constexpr (sizeof(T) == 4) { s0 = ldexpf(1.0f, a); s1 = ldexpf(1.0f, s - a); }
-    else { s0 = ldexp(1.0, a); s1 = ldexp(1.0, s - a); }
+__device__ __forceinline__ int half_exponent(int e) {
+    return sizeof(T) == 4 && e < -112 ? -112 : e;
 }
 
 template <typename T>
-__device__ __forceinline__ void split2(T x, T s0, T s1, __half &h, __half &l) {
-    const T xs = x * s0 * s1;
-    h = __float2half_rn((float)xs);
-    l = __float2half_rn((float)(xs - (T)__half2float(h)));
-}
+struct HalfScale {
+    T s0 = 1, s1 = 1;
+    HalfScale() = default;
+    __device__ __forceinline__ explicit HalfScale(int e) {   // e from half_exponent
+        const int s = kHalfShift - e;
+        if constexpr (sizeof(T) == 4) {
+            s0 = __int_as_float((s + 127) << 23);
+        } else {
+            s0 = ldexp(1.0, s / 2);
+            s1 = ldexp(1.0, s - s / 2);
+        }
+    }
+    __device__ __forceinline__ void split(T x, __half &h, __half &l) const {
+        const T xs = sizeof(T) == 4 ? x * s0 : x * s0 * s1;
+        h = __float2half_rn((float)xs);
+        l = __float2half_rn((float)(xs - (T)__half2float(h)));
+    }
+};
 
 // Fixed-point six-way split of an FP64 value (the FP64-emulation pre-pass): x' = x 2^-e
 // (|x'| < 2) is rounded to the nearest multiple of 2^-46, X = round(x' 2^46) with |X| <= 2^47,
@@ -85,6 +102,30 @@ __device__ __forceinline__ void split6(double x, int e, __nv_bfloat16 (&s)[6]) {
         X = (X - d) >> 8;
     }
     s[0] = __int2bfloat16_rn((int)X);
+}
+
+// The largest of n slots of abs-max bits (8 bytes apart), in every lane of the calling warp
+template <typename T>
+__device__ __forceinline__ T slots_max(const void *slots, uint32_t n) {
+    using U = typename std::conditional<sizeof(T) == 4, unsigned int, unsigned long long>::type;
+    U m = 0;
+    for (uint32_t i = threadIdx.x & 31; i < n; i += 32)
+        m = max(m, __ldcg(reinterpret_cast<const U *>(static_cast<const char *>(slots) + 8 * i)));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    T v;
+    memcpy(&v, &m, sizeof(T));
+    return v;
+}
+
+// exponent e with m in [2^e, 2^(e+1)); 0 for m = 0
+template <typename T>
+__device__ __forceinline__ int exponent_of(T m) {
+    if (!(m > (T)0)) return 0;
+    int e;
+    if constexpr (sizeof(T) == 4) frexpf(m, &e);
+    else frexp(m, &e);
+    return e - 1;
 }
 
 // exponent e with max|x| in [2^e, 2^(e+1)) from the abs-max bits; 0 for an all-zero (or

@@ -52,3 +52,25 @@ def test_small_rows_keep_their_relative_precision(comet):
     C, ref = run(comet, E, ext, [A, B]), oracle.einsum(E, A, B)
     rows = np.abs(C - ref).max(axis=1) / np.abs(ref).max(axis=1)
     assert rows.max() <= 1e-6
+
+
+@pytest.mark.parametrize("views", [False, True])
+@pytest.mark.parametrize("M,N,K", [(70, 50, 40), (700, 600, 300)])
+def test_scale_slots_ignore_non_finite_elements(comet, M, N, K, views):
+    # one block of the abs-max pass and many; an infinity and a NaN spoil their own rows only: the
+    # operand's scale comes from its finite elements
+    ext = dict(m=M, n=N, k=K)
+    A, B = f32((K, M), 74, 0, kind="normal"), f32((K, N), 74, 1, kind="normal")
+    A[:, 5] *= 2.0 ** 20
+    ref = oracle.einsum(E, A, B)
+    A[K // 2, 3], A[K - 1, M - 1] = np.inf, np.nan
+    kw = {}
+    if views:   # A inside a larger stored tensor of much larger values
+        S = np.full((K + 3, M + 2), 1e30, order="F")
+        S[2:K + 2, 1:M + 1] = A
+        A, kw = S, dict(views=[(0, 0, K + 3, 2, 1), (0, 1, M + 2, 1, 1)])
+    C = run(comet, E, ext, [A, B], ksplit=1, **kw)
+    fine = np.ones(M, bool)
+    fine[[3, M - 1]] = False
+    assert normwise(C[fine], ref[fine]) <= 6e-7
+    assert not np.isfinite(C[~fine]).any()
