@@ -296,7 +296,8 @@ static comet_status_t run_plan(const Plan &P, const void *const *inputs, void *o
             if (st.kernel == KK_GEMM_EMU) {
                 ProfScope ps(PK_EMU, stream);
                 e = launch_gemm_emu(g, w + st.ws_parts_a, w + st.ws_parts_b, st.kpad, sc_a, sc_b,
-                                    P.opts.debug_flags, stream, 0);
+                                    P.opts.debug_flags, stream, reinterpret_cast<long long *>(w + st.ws_ksplit),
+                                    (int64_t)st.ksplit_bytes);
                 if (e != cudaSuccess) return cuda_status(e, "emulated FP64 gemm kernel");
             } else {
                 ProfScope ps(PK_SPLIT, stream);
@@ -555,7 +556,8 @@ static comet_status_t run_host_pipe(const Plan &P, int n_calls, const void *cons
             void *sb = x_is_b ? static_cast<void *>(sc_x(j)) : static_cast<void *>(sc_w(i));
             if (emu) {
                 ProfScope ps(PK_EMU, s);
-                e = launch_gemm_emu(g, pa, pb, st.kpad, sa, sb, P.opts.debug_flags, s, 0);
+                e = launch_gemm_emu(g, pa, pb, st.kpad, sa, sb, P.opts.debug_flags, s,
+                                    reinterpret_cast<long long *>(w + st.ws_ksplit), (int64_t)st.ksplit_bytes);
             } else {
                 ProfScope ps(PK_SPLIT, s);
                 e = launch_gemm_split(g, pa, pb, st.kpad, sa, sb, (int)es, P.opts.debug_flags, s,

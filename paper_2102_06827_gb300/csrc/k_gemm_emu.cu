@@ -25,6 +25,7 @@
 //   warp 1      allocates 512 tensor-memory columns (six groups of 80); lane 0 issues the MMAs
 //   warps 2..9  epilogue: lane quadrant x half of the 80 columns; int64 sums in registers
 //   2-stage shared-memory ring (78 KB per stage).
+// Tiles beyond whole rounds over the SMs run in K slices (emu_schedule).
 // Every wait is bounded (%globaltimer); on expiry the CTA records COMET_ERR_TIMEOUT in the
 // status word, drains its own copies in flight, frees its tensor memory and returns.
 #include <cuda.h>
@@ -35,12 +36,13 @@
 #include "launch.h"
 #include "params.h"
 #include "sm100.cuh"
+#include "split_schedule.h"
 
 namespace comet {
 
 namespace emu {
 constexpr int S = 6;                            // slices per operand
-constexpr int BM = 128, BG = 80, BK = 32, STAGES = 2;
+constexpr int BM = kEmuBM, BG = kEmuBN, BK = 32, STAGES = 2;
 constexpr int A_PLANE = BM * BK * 2;            // 8 KB
 constexpr int B_PLANE = BG * BK * 2;            // 5 KB
 constexpr int A_STAGE = S * A_PLANE;            // 48 KB
@@ -54,13 +56,19 @@ static_assert(GROUPS * BG <= (int)TMEM_COLS, "every weight group's accumulator i
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align*/ + BG * 8 /*c_col*/ + 256;
 constexpr uint32_t SW64 = 4;
 constexpr uint32_t SBO = 8 * BK * 2;
-constexpr uint32_t KC_BLOCKS = 6;               // 192 K values per exact chunk
+constexpr uint32_t KC_BLOCKS = kEmuChunk / BK;  // 192 K values per exact chunk
 constexpr uint32_t MAX_K = 96 * 1024;           // keeps the int64 sums below 2^63
 constexpr int HALF = BG / 2;                    // columns per epilogue thread
 }  // namespace emu
 
 struct EmuArgs {
     uint32_t m_tiles, n_tiles, nkb;
+    uint32_t full, tail, slices; // items: `full` whole tiles, then slices x tail items (K slices of the
+                                 // tiles from `full` on)
+    uint32_t slice_blocks;       // K blocks per slice (a multiple of the chunk's)
+    uint32_t items;
+    long long *partial;          // [slice][tail tile][column][row] int64 sums
+    DbgRange dbg_p;              // debug builds: their buffer
     int debug_flags;
     const void *scale_a;         // bits of max |A|, max |B| (FP64)
     const void *scale_b;
@@ -72,6 +80,18 @@ __device__ __forceinline__ int exp_of_max_f64(const void *bits) {
     int e;
     frexp(m, &e);
     return e - 1;
+}
+
+// tile -> (m tile, n tile): bands of 16 m-tiles, n-major inside a band, for L2 reuse
+__device__ __forceinline__ void emu_tile_coords(uint32_t t, uint32_t m_tiles, uint32_t n_tiles, uint32_t &mt,
+                                                uint32_t &nt) {
+    const uint32_t G = 16;
+    const uint32_t band = t / (G * n_tiles);
+    const uint32_t base = band * G;
+    const uint32_t g = min(G, m_tiles - base);
+    const uint32_t r = t - band * G * n_tiles;
+    mt = base + r % g;
+    nt = r / g;
 }
 
 __global__ void __launch_bounds__(emu::THREADS, 1)
@@ -92,7 +112,6 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t tmo = (uint64_t)p.timeout_ns;
-    const uint32_t n_tiles_total = x.m_tiles * x.n_tiles;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -115,15 +134,19 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
         *abort_flag = 1;
         atomicExch(p.status, (int)COMET_ERR_TIMEOUT);
     };
-    // tile t -> (m tile, n tile): bands of 16 m-tiles, n-major inside a band, for L2 reuse
-    auto tile_coords = [&](uint32_t t, uint32_t &mt, uint32_t &nt) {
-        const uint32_t G = 16;
-        uint32_t band = t / (G * x.n_tiles);
-        uint32_t base = band * G;
-        uint32_t g = min(G, x.m_tiles - base);
-        uint32_t r = t - band * G * x.n_tiles;
-        mt = base + r % g;
-        nt = r / g;
+    // item t -> its tile and K blocks kb0 .. kb1 - 1; true for a K slice
+    auto item = [&](uint32_t t, uint32_t &mt, uint32_t &nt, uint32_t &kb0, uint32_t &kb1) {
+        kb0 = 0;
+        kb1 = x.nkb;
+        const bool sliced = t >= x.full;
+        if (sliced) {
+            const uint32_t u = t - x.full, ks = u / x.tail;
+            t = x.full + (u - ks * x.tail);
+            kb0 = ks * x.slice_blocks;
+            kb1 = min(x.nkb, kb0 + x.slice_blocks);
+        }
+        emu_tile_coords(t, x.m_tiles, x.n_tiles, mt, nt);
+        return sliced;
     };
 
     if (warp == 0) {
@@ -132,10 +155,10 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
             uint32_t it = 0;
             bool ok = true;
             bool injected = false;
-            for (uint32_t t = blockIdx.x; t < n_tiles_total && ok; t += gridDim.x) {
-                uint32_t mt, nt;
-                tile_coords(t, mt, nt);
-                for (uint32_t kb = 0; kb < x.nkb; ++kb, ++it) {
+            for (uint32_t t = blockIdx.x; t < x.items && ok; t += gridDim.x) {
+                uint32_t mt, nt, kb0, kb1;
+                item(t, mt, nt, kb0, kb1);
+                for (uint32_t kb = kb0; kb < kb1; ++kb, ++it) {
                     const uint32_t s = it % STAGES, round = it / STAGES;
                     if (round > 0 && !mbar_wait(&empty[s], (round - 1) & 1, tmo, abort_flag)) {
                         fail(); ok = false; break;
@@ -164,9 +187,11 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
             auto G = [&](int w) { return tmem_base + (uint32_t)(w * BG); };
             uint32_t it = 0, chunk = 0;
             bool ok = true;
-            for (uint32_t t = blockIdx.x; t < n_tiles_total && ok; t += gridDim.x) {
-                for (uint32_t kb = 0; kb < x.nkb; ++kb, ++it) {
-                    const uint32_t kin = kb % KC_BLOCKS;
+            for (uint32_t t = blockIdx.x; t < x.items && ok; t += gridDim.x) {
+                uint32_t mt, nt, kb0, kb1;
+                item(t, mt, nt, kb0, kb1);
+                for (uint32_t kb = kb0; kb < kb1; ++kb, ++it) {
+                    const uint32_t kin = kb % KC_BLOCKS;   // slices start on chunk boundaries
                     if (kin == 0) {
                         if (chunk > 0 && !mbar_wait(tempty, (chunk - 1) & 1, tmo, abort_flag)) {
                             fail(); ok = false; break;
@@ -195,7 +220,7 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
                         mma_bf16(G(5), a(5), b(0), id1, 1);   // group 5
                     }
                     mma_commit(&empty[s]);
-                    if (kin == KC_BLOCKS - 1 || kb == x.nkb - 1) {
+                    if (kin == KC_BLOCKS - 1 || kb == kb1 - 1) {
                         mma_commit(tfull);
                         ++chunk;
                     }
@@ -212,13 +237,13 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
         const int e_sum = exp_of_max_f64(x.scale_a) + exp_of_max_f64(x.scale_b);
         const double scale = ldexp(p.alpha, e_sum - 44);
-        const uint32_t nchunks = (x.nkb + KC_BLOCKS - 1) / KC_BLOCKS;
         uint32_t chunk = 0;
         bool dead = false;
         double *C = reinterpret_cast<double *>(p.C);
-        for (uint32_t t = blockIdx.x; t < n_tiles_total; t += gridDim.x) {
-            uint32_t mt, nt;
-            tile_coords(t, mt, nt);
+        for (uint32_t t = blockIdx.x; t < x.items; t += gridDim.x) {
+            uint32_t mt, nt, kb0, kb1;
+            const bool sliced = item(t, mt, nt, kb0, kb1);
+            const uint32_t nchunks = (kb1 - kb0 + KC_BLOCKS - 1) / KC_BLOCKS;
             named_bar_sync(1, 32 * EPI_WARPS);
             if (et < BG) {
                 int64_t o0 = 0, o1 = 0;
@@ -283,7 +308,12 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
             }
             if (dead) continue;
             const uint32_t m = mt * BM + quad * 32 + lane;
-            if (m < p.M) {
+            if (sliced) {   // the slice's sums to its slot, row fastest (coalesced)
+                long long *P = x.partial + ((size_t)(t - x.full) * BG + half * HALF) * BM + quad * 32 + lane;
+#pragma unroll
+                for (int j = 0; j < HALF; ++j)
+                    if (dbg_ok(x.dbg_p, P + (size_t)j * BM, 8, p.status)) P[(size_t)j * BM] = I[j];
+            } else if (m < p.M) {
                 int64_t r0 = 0, c_row = 0;
                 radix_offsets(p.ma, m, r0, c_row);
                 const uint32_t n_valid = min((uint32_t)BG, p.N - nt * BG);
@@ -310,6 +340,41 @@ __global__ void __launch_bounds__(emu::THREADS, 1)
     __syncthreads();
     tc_fence_after();
     if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
+}
+
+// K-slice partials -> C for the tail tiles; a block takes 16 columns of a tile, a thread one row and
+// eight of the columns
+__global__ void __launch_bounds__(256) emu_reduce_kernel(const GemmParams p, const EmuArgs x) {
+    using namespace emu;
+    constexpr int STRIP = 16;
+    __shared__ int64_t c_col[STRIP];
+    const uint32_t jt = blockIdx.x / (BG / STRIP), strip = blockIdx.x % (BG / STRIP);
+    uint32_t mt, nt;
+    emu_tile_coords(x.full + jt, x.m_tiles, x.n_tiles, mt, nt);
+    const uint32_t ml = threadIdx.x & (BM - 1), m = mt * BM + ml, n0 = nt * BG + strip * STRIP;
+    if (threadIdx.x < STRIP && n0 + threadIdx.x < p.N) {
+        int64_t o0, o1;
+        radix_offsets(p.nb, n0 + threadIdx.x, o0, o1);
+        c_col[threadIdx.x] = o1;
+    }
+    int64_t r0 = 0, c_row = 0;
+    if (m < p.M) radix_offsets(p.ma, m, r0, c_row);
+    pdl_wait();
+    __syncthreads();
+    if (m >= p.M) return;
+    const double scale = ldexp(p.alpha, exp_of_max_f64(x.scale_a) + exp_of_max_f64(x.scale_b) - 44);
+    for (uint32_t j = threadIdx.x / BM; j < STRIP; j += 256 / BM) {
+        if (n0 + j >= p.N) break;
+        long long sum = 0;
+        for (uint32_t k = 0; k < x.slices; ++k) {
+            const long long *q = x.partial + (((size_t)k * x.tail + jt) * BG + strip * STRIP + j) * BM + ml;
+            if (dbg_ok(x.dbg_p, q, 8, p.status)) sum += *q;
+        }
+        double *dst = reinterpret_cast<double *>(p.C) + c_row + c_col[j];
+        if (!dbg_ok(p.dbg_c, dst, 8, p.status)) continue;
+        const double v = scale * (double)sum;
+        *dst = p.beta != 0.0 ? v + p.beta * *dst : v;
+    }
 }
 
 // ---- host side --------------------------------------------------------------------------------
@@ -357,7 +422,7 @@ static int sm_count_emu() {
 
 cudaError_t launch_gemm_emu(const GemmParams &p, const void *parts_a, const void *parts_b, int64_t kpad,
                             const void *scale_a, const void *scale_b, int debug_flags, cudaStream_t s,
-                            int max_ctas) {
+                            long long *partial, int64_t partial_bytes) {
     using namespace emu;
     if (p.M == 0 || p.N == 0) return cudaSuccess;
     if (p.K > MAX_K) return cudaErrorInvalidValue;
@@ -371,16 +436,26 @@ cudaError_t launch_gemm_emu(const GemmParams &p, const void *parts_a, const void
     x.debug_flags = debug_flags;
     x.scale_a = scale_a;
     x.scale_b = scale_b;
-    const uint32_t tiles = x.m_tiles * x.n_tiles;
-    int ctas = sm_count_emu();
-    if (max_ctas > 0 && max_ctas < ctas) ctas = max_ctas;
-    if ((uint32_t)ctas > tiles) ctas = (int)tiles;
+    const uint32_t sms = (uint32_t)sm_count_emu();
+    const EmuSchedule sch = emu_schedule(p.M, p.N, p.K, sms, partial ? partial_bytes : 0);
+    x.full = sch.full;
+    x.tail = sch.tail;
+    x.slices = sch.slices;
+    x.items = sch.full + sch.tail * sch.slices;
+    const uint32_t nch = (x.nkb + KC_BLOCKS - 1) / KC_BLOCKS;
+    x.slice_blocks = (nch + sch.slices - 1) / sch.slices * KC_BLOCKS;
+    x.partial = partial;
+    x.dbg_p = dbg_range(partial, emu_partial_bytes(sch));
+    const int ctas = (int)std::min(sms, x.items);
     static bool attr_set = false;
     if (!attr_set) {
         cudaFuncSetAttribute(gemm_emu_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
         attr_set = true;
     }
     launch_pdl(gemm_emu_kernel, ctas, THREADS, SMEM_BYTES, s, ta, tb, p, x);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || x.slices == 1) return e;
+    launch_pdl(emu_reduce_kernel, x.tail * (BG / 16), 256, 0, s, p, x);
     return cudaGetLastError();
 }
 

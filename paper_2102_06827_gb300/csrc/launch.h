@@ -74,9 +74,10 @@ cudaError_t launch_gemm_split(const GemmParams &p, const void *parts_a, const vo
                               int out_bytes, int debug_flags, cudaStream_t s,
                               uint32_t want_ksplit, float *partial, int64_t partial_bytes);
 
+// `partial`: room for the int64 sums of K slices (emu_schedule; as many as fit partial_bytes)
 cudaError_t launch_gemm_emu(const GemmParams &p, const void *parts_a, const void *parts_b, int64_t kpad,
                             const void *scale_a, const void *scale_b, int debug_flags, cudaStream_t s,
-                            int max_ctas);
+                            long long *partial, int64_t partial_bytes);
 
 cudaError_t launch_gemv(const GemvParams &p, int elem_bytes, cudaStream_t s);
 

@@ -1061,17 +1061,24 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
         st.ws_parts_a = parts_base;
         st.ws_parts_b = parts_base + ba;
         size_t bk = 0, least = 0;
+        // Partial sums of K slices stay inside the library's static scratch when the plan without them
+        // does, else within 256 MB.
+        const int64_t fixed = COMET_NOALLOC_MAX_BYTES - 256 - 16 * kSlots;
+        auto room_for = [&](size_t without) {
+            return (int64_t)(parts_base + without) <= fixed ? (fixed - (int64_t)(parts_base + ba + bb)) / 256 * 256
+                                                            : (int64_t)256 << 20;
+        };
+        if (st.kernel == KK_GEMM_EMU) {
+            const EmuSchedule sch = emu_schedule((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, 152, room_for(ba + bb));
+            bk = (size_t)emu_partial_bytes(sch);
+        }
         if (st.kernel == KK_GEMM_SPLIT) {
-            // tile width and K slices (split_schedule).  The partial sums stay inside the library's
-            // static scratch when the plan without them would (three planes per operand were
-            // kept before; the step's room is never less than theirs), else within 256 MB
+            // tile width and K slices (split_schedule); the step's room is never less than the three planes
+            // per operand that were kept before
             least = align((size_t)6 * rows_a * st.kpad) + align((size_t)6 * rows_b * st.kpad);
-            const int64_t fixed = COMET_NOALLOC_MAX_BYTES - 256 - 16 * kSlots;
-            const int64_t limit = (int64_t)(parts_base + least) <= fixed ? fixed - (int64_t)(parts_base + ba + bb)
-                                                                         : (int64_t)256 << 20;
             st.want_ksplit = opts.ksplit > 0 ? (uint32_t)opts.ksplit : 0;
             const SplitSchedule sch = split_schedule((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, 76,
-                                                     st.want_ksplit, limit / 256 * 256);
+                                                     st.want_ksplit, room_for(least));
             st.ksplit = sch.ksplit;
             st.tile_n = sch.bn;
             // one launch on the FP32 pipes where that is modelled faster than the split form's chain

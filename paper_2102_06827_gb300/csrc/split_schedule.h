@@ -80,4 +80,42 @@ inline double small_gemm_us(uint64_t M, uint64_t N, uint64_t K, bool long_runs) 
     return 3.0 + (double)((tiles + 151) / 152) * (900.0 + (double)K * (long_runs ? 22.0 : 42.0)) / 1900.0;
 }
 
+// The emulated-FP64 GEMM: whole-K tiles of 128 x 80 in full waves over the SMs, the tiles left over in
+// K slices of whole chunks (192 values) whose int64 partial sums a second kernel adds.
+constexpr int kEmuBM = 128, kEmuBN = 80, kEmuChunk = 192;
+
+struct EmuSchedule {
+    uint32_t full = 0;      // tiles computed whole
+    uint32_t tail = 0;      // tiles left over
+    uint32_t slices = 1;    // K slices of each of them (1: whole as well)
+};
+
+inline int64_t emu_partial_bytes(const EmuSchedule &s) {
+    return s.slices > 1 ? (int64_t)s.tail * s.slices * kEmuBM * kEmuBN * 8 : 0;
+}
+
+// The slices of the left-over tiles that end soonest, in units of a chunk's time (about 8 us): rounds
+// over the SMs times chunks per slice plus 0.4 around each item, plus 0.5 for the second kernel.
+// At 1728^3 (308 tiles, nine chunks) the four tiles after two rounds of 152 run in 36 slices on idle SMs
+// instead of a third round.  Chunks keep their boundaries and the sums are integers, so slicing
+// changes no bit of the result.
+inline EmuSchedule emu_schedule(uint64_t M, uint64_t N, uint64_t K, uint32_t sms, int64_t partial_limit) {
+    const uint32_t tiles = (uint32_t)(((M + kEmuBM - 1) / kEmuBM) * ((N + kEmuBN - 1) / kEmuBN));
+    const uint32_t nch = (uint32_t)std::max<uint64_t>(1, (K + kEmuChunk - 1) / kEmuChunk);
+    EmuSchedule s, best;
+    s.full = tiles / sms * sms;
+    s.tail = tiles - s.full;
+    best.full = tiles;
+    if (s.tail == 0) return best;
+    double least = (double)nch + 0.4;
+    for (uint32_t k = 2; k <= std::min(nch, 32u); ++k) {
+        const uint32_t per = (nch + k - 1) / k;
+        s.slices = (nch + per - 1) / per;
+        if (emu_partial_bytes(s) > partial_limit) break;
+        const double t = (double)((s.tail * s.slices + sms - 1) / sms) * (per + 0.4) + 0.5;
+        if (t < least) { least = t; best = s; }
+    }
+    return best;
+}
+
 }  // namespace comet
