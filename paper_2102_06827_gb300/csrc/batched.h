@@ -55,7 +55,8 @@ struct BatchedParams {
     void *result;
     uint32_t key;
     unsigned int *counter;       // work counter (zeroed by the launch sequence)
-    const int *exps;             // split path: scale exponents of the M and N operands, 2 per block
+    int *exps;                   // split path: scale exponents of the M and N operands, 2 per block, as
+                                 // batched_exp reads them (zeroed by the launch sequence)
     double alpha;
     char *ws;                    // workspace base
     char *planes;                // split path: start of the plane region
@@ -64,6 +65,12 @@ struct BatchedParams {
     int64_t timeout_ns;          // limit of every wait of the tensor-core kernel
     int debug_flags;             // bit 0: one operand load withheld (fault injection, host side)
 };
+
+// An operand's exponent word: 0 = no non-zero element seen, kExpNonFinite = a non-finite one, else
+// the exponent of the largest magnitude seen + kExpBias.  The order of the words is the order in which
+// one replaces another, so that the CTAs of an operand combine theirs with one atomic maximum each.
+constexpr int kExpBias = 4096, kExpNonFinite = 1 << 20;
+CM_HD int batched_exp(int word) { return word == 0 || word >= kExpNonFinite ? 0 : word - kExpBias; }
 
 // tile configurations: rows x columns of a work item's tiles (the split path's rows are the
 // tcgen05 M; its columns are the strip width of a work item)
@@ -75,6 +82,12 @@ inline TileCfg batched_cfg(bool split, int c) {
 }
 inline int n_cfg(const Plan &P) { return P.opts.precision == COMET_PREC_SPLIT_BF16 ? kBatchedCfgSplit : kBatchedCfgF64; }
 inline TileCfg cfg_of(const Plan &P, int c) { return batched_cfg(P.opts.precision == COMET_PREC_SPLIT_BF16, c); }
+
+// CTAs per operand of the pre-passes: about 16 per SM over the whole grid, at most 64
+inline uint32_t batched_shares(int n_blocks) {
+    const int64_t want = (152 * 16 + 2 * (int64_t)n_blocks - 1) / (2 * (int64_t)n_blocks);
+    return (uint32_t)(want < 1 ? 1 : want > 64 ? 64 : want);
+}
 
 // workspace layout: [counter 256 B][exps 8*n][prefix n_cfg*(n+1)*4][descs n*sizeof(BlockDesc)]
 // [split path: item records of every configuration][split path: the plane rows of every

@@ -239,7 +239,9 @@ __global__ void __launch_bounds__(BT) batched_f64_kernel(const BatchedParams P) 
     }
 }
 
-// per-block operand scale exponents (split path): CTA c reduces operand c%2 of block c/2.
+// per-block operand scale exponents (split path): CTA (c, y) reduces a share of operand c%2 of block
+// c/2 (grid.y shares: one CTA per operand left the largest one, 1 M elements, to 366 us of scalar
+// loads while the others were done).
 // The largest magnitude is taken on the bit patterns with the sign bit cleared (for finite
 // values the unsigned integer order is the order of magnitudes), so the reduction is exact
 // and runs on the integer pipe for both input precisions.
@@ -252,16 +254,10 @@ __global__ void __launch_bounds__(256) batched_absmax_kernel(const BatchedParams
     const int op = blockIdx.x & 1;
     const int64_t n = op ? d.b_elems : d.a_elems;
     const U *x = reinterpret_cast<const U *>(P.inputs[2 * d.index + (op ^ P.swap)]);
-    U m0 = 0, m1 = 0, m2 = 0, m3 = 0;
-    int64_t i = threadIdx.x;
-    for (; i + 3 * 256 < n; i += 4 * 256) {
-        m0 = max(m0, x[i] & MAG);
-        m1 = max(m1, x[i + 256] & MAG);
-        m2 = max(m2, x[i + 512] & MAG);
-        m3 = max(m3, x[i + 768] & MAG);
-    }
-    for (; i < n; i += 256) m0 = max(m0, x[i] & MAG);
-    U m = max(max(m0, m1), max(m2, m3));
+    U m = 0;
+    const int64_t step = (int64_t)gridDim.y * 256;
+#pragma unroll 8
+    for (int64_t i = (int64_t)blockIdx.y * 256 + threadIdx.x; i < n; i += step) m = max(m, x[i] & MAG);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, (U)__shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
@@ -269,16 +265,17 @@ __global__ void __launch_bounds__(256) batched_absmax_kernel(const BatchedParams
     if (threadIdx.x == 0) {
         U mm = 0;
         for (int w = 0; w < 8; ++w) mm = max(mm, red[w]);
-        // exponent e with max |x| in [2^e, 2^(e+1)); 0 for an all-zero or non-finite operand
-        int e = 0;
+        if (mm == 0) return;
+        // exponent e with max |x| in [2^e, 2^(e+1))
+        int e = 0, word = kExpNonFinite;
         if constexpr (sizeof(TIn) == 4) {
             const float v = __uint_as_float((uint32_t)mm);
-            if (v > 0.0f && !isinf(v) && !isnan(v)) { frexpf(v, &e); e -= 1; }
+            if (!isinf(v) && !isnan(v)) { frexpf(v, &e); word = e - 1 + kExpBias; }
         } else {
             const double v = __longlong_as_double((long long)mm);
-            if (v > 0.0 && !isinf(v) && !isnan(v)) { frexp(v, &e); e -= 1; }
+            if (!isinf(v) && !isnan(v)) { frexp(v, &e); word = e - 1 + kExpBias; }
         }
-        const_cast<int *>(P.exps)[2 * d.index + op] = e;
+        atomicMax(P.exps + 2 * d.index + op, word);
     }
 }
 
@@ -333,7 +330,7 @@ static comet_status_t run_batched(const Plan &P, const void *const *block_inputs
     bp.result = result;
     bp.key = key;
     bp.counter = reinterpret_cast<unsigned int *>(w);
-    bp.exps = reinterpret_cast<const int *>(w + L.exps);
+    bp.exps = reinterpret_cast<int *>(w + L.exps);
     bp.alpha = P.alpha;
     bp.ws = w;
     bp.planes = w + L.parts;
@@ -344,13 +341,16 @@ static comet_status_t run_batched(const Plan &P, const void *const *block_inputs
     bp.timeout_ns = (P.opts.timeout_ms > 0 ? P.opts.timeout_ms : 2000) * 1000000ll;
     bp.debug_flags = P.opts.debug_flags;
     if (!bp.status) return COMET_ERR_CUDA;
-    cudaError_t e = cudaMemsetAsync(w, 0, 16, s);
+    // the work counter, and with the split path the exponent words behind it
+    const bool split = P.opts.precision == COMET_PREC_SPLIT_BF16;
+    cudaError_t e = cudaMemsetAsync(w, 0, split ? L.exps + 8 * (size_t)P.n_blocks : 16, s);
     if (e == cudaSuccess && mode == 0) e = cudaMemsetAsync(result, 0, 16 * (size_t)P.n_blocks, s);
     if (e != cudaSuccess) return COMET_ERR_CUDA;
-    if (P.opts.precision == COMET_PREC_SPLIT_BF16) {
+    if (split) {
         int h = prof_begin(PK_BATCHED_PREPASS_ID, s);
-        if (P.dtype == COMET_F32) batched_absmax_kernel<float><<<2 * nb, 256, 0, s>>>(bp);
-        else batched_absmax_kernel<double><<<2 * nb, 256, 0, s>>>(bp);
+        const dim3 grid(2 * nb, batched_shares(nb));
+        if (P.dtype == COMET_F32) batched_absmax_kernel<float><<<grid, 256, 0, s>>>(bp);
+        else batched_absmax_kernel<double><<<grid, 256, 0, s>>>(bp);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = launch_batched_presplit(bp, nb, P.dtype == COMET_F64, s);
         prof_end(h, s);

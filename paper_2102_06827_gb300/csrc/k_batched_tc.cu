@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(btc::THREADS, 1)
             const BlockDesc *d = P.desc + cur.pos;
             const uint32_t M = cur.M, N = cur.N, idx = cur.index, mtiles = cur.mtiles, n0 = cur.n0;
             const uint32_t hb = idx * 0x9E3779B9u;
-            const int e_sum = P.exps[2 * idx] + P.exps[2 * idx + 1];
+            const int e_sum = batched_exp(P.exps[2 * idx]) + batched_exp(P.exps[2 * idx + 1]);
             // the strip's column offsets and weight factors, and the block's row digits in shared
             // memory (all eight warps meet here)
             named_bar_sync(1, 32 * EPI_WARPS);
@@ -462,9 +462,12 @@ __global__ void __launch_bounds__(btc::THREADS, 1)
     if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
 }
 
-// Split pre-pass: CTA c writes operand c%2 of block c/2 (launch order) as plane rows
+// Split pre-pass: CTA (c, y) writes a share of operand c%2 of block c/2 (launch order) as plane rows
 // [chunk][plane][row] of 32 K values, rows to the operand's padded row count, scaled by the
-// block's exponent; one thread per row, 64 bytes per plane row (coalesced across the warp).
+// block's exponent.  Four threads per row, each eight K values and 16 bytes of every plane row, so
+// that a warp's stores are whole 512-byte runs and its loads either run along eight rows or along
+// K.  256 blocks, 0.37 GB read and 0.75 GB written (165 us of HBM): 509 us with one thread per row and
+// one CTA per operand, 306 in shares (grid.y), 220 now.
 template <typename TIn>
 __global__ void __launch_bounds__(256) batched_presplit_tc_kernel(const BatchedParams P) {
     __shared__ int64_t k_off[1024];
@@ -475,7 +478,7 @@ __global__ void __launch_bounds__(256) batched_presplit_tc_kernel(const BatchedP
     const TIn *x = reinterpret_cast<const TIn *>(P.inputs[2 * d.index + (op ^ P.swap)]);
     const DbgRange xr = dbg_range(x, (op ? d.b_elems : d.a_elems) * (int64_t)sizeof(TIn));
     const DbgRange pr = dbg_range(P.planes, P.planes_bytes);
-    const int e = P.exps[2 * d.index + op];
+    const int e = batched_exp(P.exps[2 * d.index + op]);
     uint4 *base = reinterpret_cast<uint4 *>(P.planes + (op ? d.b_row0 : d.a_row0) * kBatchedPlaneRow);
     for (uint32_t k = threadIdx.x; k < nkc * 32; k += 256) {
         int64_t o0 = 0, o1 = 0;
@@ -483,35 +486,49 @@ __global__ void __launch_bounds__(256) batched_presplit_tc_kernel(const BatchedP
         k_off[k] = op ? o1 : o0;
     }
     __syncthreads();
-    for (uint32_t r = threadIdx.x; r < pad; r += 256) {
-        int64_t ro = 0, o1 = 0;
-        const bool valid = r < rows;
-        if (valid) radix_offsets(rr, r, ro, o1);
-        for (uint32_t kc = 0; kc < nkc; ++kc) {
+    const float s0 = ldexpf(1.0f, -e / 2), s1 = ldexpf(1.0f, -e - (-e / 2));
+    const uint32_t lane = threadIdx.x & 31, q = lane & 3;   // q: eight of the chunk's 32 K values
+    // a warp takes 32 rows: each lane works out one row's offset, then eight rows at a time
+    for (uint32_t r32 = (blockIdx.y * 8 + threadIdx.x / 32) * 32; r32 < pad; r32 += gridDim.y * 256) {
+        int64_t mine = 0, o1 = 0;
+        if (r32 + lane < rows) radix_offsets(rr, r32 + lane, mine, o1);
+        for (uint32_t it = 0; it < 4 * nkc; ++it) {
+            const uint32_t kc = it >> 2, sub = (it & 3) * 8 + lane / 4, r = r32 + sub;
+            const int64_t ro = __shfl_sync(0xffffffffu, mine, sub);
+            const bool valid = r < rows;
+            const uint32_t k0 = kc * 32 + q * 8;
+            TIn v[8];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {   // 16 K values (32 bytes) per plane at a time
-                uint32_t w[3][8];
+            for (int j = 0; j < 8; ++j) {
+                const TIn *src = x + ro + k_off[k0 + j];
+                v[j] = valid && k0 + j < K && dbg_ok(xr, src, (int)sizeof(TIn), P.status) ? *src : (TIn)0;
+            }
+            uint32_t w[3][4];
 #pragma unroll
-                for (int j = 0; j < 16; j += 2) {
-                    __nv_bfloat16 h0, m0, l0, h1, m1, l1;
-                    const uint32_t k = kc * 32 + half * 16 + j;
-                    const TIn v0 = (valid && k < K && dbg_ok(xr, x + ro + k_off[k], (int)sizeof(TIn), P.status))
-                                       ? x[ro + k_off[k]] : (TIn)0;
-                    const TIn v1 = (valid && k + 1 < K && dbg_ok(xr, x + ro + k_off[k + 1], (int)sizeof(TIn), P.status))
-                                       ? x[ro + k_off[k + 1]] : (TIn)0;
-                    split3<TIn>(v0, e, h0, m0, l0);
-                    split3<TIn>(v1, e, h1, m1, l1);
-                    w[0][j >> 1] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-                    w[1][j >> 1] = (uint32_t)__bfloat16_as_ushort(m0) | ((uint32_t)__bfloat16_as_ushort(m1) << 16);
-                    w[2][j >> 1] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+            for (int j = 0; j < 4; ++j) {
+                float f[2][3];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if constexpr (sizeof(TIn) == 4) {
+                        split3_floats(v[2 * j + u], s0, s1, f[u][0], f[u][1], f[u][2]);
+                    } else {
+                        __nv_bfloat16 h, m, l;
+                        split3<TIn>(v[2 * j + u], e, h, m, l);
+                        f[u][0] = __bfloat162float(h);
+                        f[u][1] = __bfloat162float(m);
+                        f[u][2] = __bfloat162float(l);
+                    }
                 }
 #pragma unroll
                 for (int p = 0; p < 3; ++p) {
-                    uint4 *dst = base + ((size_t)(kc * 3 + p) * pad + r) * 4 + half * 2;
-                    if (!dbg_ok(pr, dst, 32, P.status)) continue;
-                    dst[0] = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
-                    dst[1] = make_uint4(w[p][4], w[p][5], w[p][6], w[p][7]);
+                    const __nv_bfloat162 pair = __floats2bfloat162_rn(f[0][p], f[1][p]);
+                    w[p][j] = *reinterpret_cast<const uint32_t *>(&pair);
                 }
+            }
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                uint4 *dst = base + ((size_t)(kc * 3 + p) * pad + r) * 4 + q;
+                if (dbg_ok(pr, dst, 16, P.status)) *dst = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
             }
         }
     }
@@ -536,8 +553,9 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 cudaError_t launch_batched_presplit(const BatchedParams &bp, int n_blocks, bool f64_in, cudaStream_t s) {
     if (n_blocks <= 0) return cudaSuccess;
-    if (f64_in) batched_presplit_tc_kernel<double><<<2 * n_blocks, 256, 0, s>>>(bp);
-    else batched_presplit_tc_kernel<float><<<2 * n_blocks, 256, 0, s>>>(bp);
+    const dim3 grid(2 * n_blocks, batched_shares(n_blocks));
+    if (f64_in) batched_presplit_tc_kernel<double><<<grid, 256, 0, s>>>(bp);
+    else batched_presplit_tc_kernel<float><<<grid, 256, 0, s>>>(bp);
     return cudaGetLastError();
 }
 

@@ -41,6 +41,21 @@ __device__ __forceinline__ void split3(T x, int e, __nv_bfloat16 &h, __nv_bfloat
     }
 }
 
+// split3 of an FP32 value as floats, for packing two of each part with one conversion: the same
+// parts bit for bit, with the scale 2^-e as a product of two normal powers of two (a scaled value
+// below 2^-126 rounds to nothing in every part) and rounding to an integer by adding and subtracting
+// 1.5 * 2^23 (valid to 2^22; the values stay below 2^8), which keep ldexpf's and rintf's
+// instructions out of the batched pre-pass.
+__device__ __forceinline__ void split3_floats(float x, float s0, float s1, float &h, float &m, float &l) {
+    constexpr float kMagic = 12582912.0f;
+    const float xs = x * s0 * s1;
+    h = __fsub_rn(__fadd_rn(xs * 64.0f, kMagic), kMagic) * (1.0f / 64.0f);
+    const float r1 = xs - h;
+    m = __fsub_rn(__fadd_rn(r1 * 16384.0f, kMagic), kMagic) * (1.0f / 16384.0f);
+    const float r2 = r1 - m;
+    l = __fsub_rn(__fadd_rn(r2 * 4194304.0f, kMagic), kMagic) * (1.0f / 4194304.0f);
+}
+
 // Two-part FP16 split of the split GEMM's pre-pass: x 2^(14-e) = h + l up to half a unit of l, h
 // and l each the nearest FP16 value to what is left (kHalfShift = 14 puts the operand's largest
 // magnitude into [2^14, 2^15), so that the exponent range of FP16 lies below it).  The residual
