@@ -194,6 +194,13 @@ constexpr int nth_label(int mask, int i) {
     return -1;
 }
 
+// (hi, lo) += (h, l): hi rounded, its exact error in lo
+__device__ __forceinline__ void add_exact(float &hi, float &lo, float h, float l) {
+    const float s = __fadd_rn(hi, h), z = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(l, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, z)), __fsub_rn(h, z))));
+    hi = s;
+}
+
 // one drain warp's 16 columns of a term's product for this thread's row: column n = 16 colq +
 // c0 + 4 c1 sits at the narrow labels' coordinates (c0, c1, colq); the first term stores, the
 // others add (all loads before the stores: the 16 slots are distinct)
@@ -228,9 +235,11 @@ __device__ __forceinline__ void drain_dispatch(int mn, float *T, int row, int co
 
 }  // namespace
 
-// Pre-pass: CTA c writes operand c % 2 of term (c / 2) % n_terms of block b0 + c / (2 n_terms),
-// one thread per plane row of the tile-blocked layout, 64 bytes per plane (coalesced across the
-// warp); rows and summed indices outside the block are zero.
+// Pre-pass: CTA (c, y) writes a share of operand c % 2 of term (c / 2) % n_terms of block
+// b0 + c / (2 n_terms); rows and summed indices outside the block are zero.  A warp takes 32 plane rows of
+// the tile-blocked layout, each lane working out one row's offset; then four lanes per row, eight summed
+// indices and 16 bytes of every plane each, so that stores are whole 512-byte runs (16 blocks: 395 us
+// with one CTA per operand and one thread per row, 173 now).
 __global__ void __launch_bounds__(256) triples_tc_split_kernel(const Args a, const TcArgs t) {
     const int seg = blockIdx.x, side = seg & 1, p = (seg >> 1) % a.n_terms;
     const int b = t.b0 + seg / (2 * a.n_terms);
@@ -241,40 +250,45 @@ __global__ void __launch_bounds__(256) triples_tc_split_kernel(const Args a, con
     const DbgRange xr = dbg_range(x, (int64_t)g.ext[0] * g.ext[1] * g.ext[2] * g.ed * 4);
     const DbgRange pr = dbg_range(t.planes, t.planes_bytes);
     const int64_t rows = (int64_t)g.nt[0] * g.nt[1] * g.nt[2] * g.rpt;
-    for (int64_t R = threadIdx.x; R < rows; R += blockDim.x) {
-        const int64_t tile = R / g.rpt;
-        const int rr = (int)(R - tile * g.rpt);
-        const int t0 = (int)(tile % g.nt[0]), t1 = (int)((tile / g.nt[0]) % g.nt[1]), t2 = (int)(tile / ((int64_t)g.nt[0] * g.nt[1]));
-        int c0, c1, c2;
-        row_coords(g.wide, rr, c0, c1, c2);
-        const int g0 = t0 * g.ts[0] + c0, g1 = t1 * g.ts[1] + c1, g2 = t2 * g.ts[2] + c2;
-        const bool valid = g0 < g.ext[0] && g1 < g.ext[1] && g2 < g.ext[2];
-        const int64_t ro = valid ? (int64_t)g0 * g.st[0] + (int64_t)g1 * g.st[1] + (int64_t)g2 * g.st[2] : 0;
-        for (int ch = 0; ch < g.nch; ++ch) {
+    const int lane = threadIdx.x & 31, q = lane & 3;
+    for (int64_t R32 = ((int64_t)blockIdx.y * 8 + threadIdx.x / 32) * 32; R32 < rows; R32 += (int64_t)gridDim.y * 256) {
+        int64_t ro_mine = -1;   // element offset of row R32 + lane; -1 outside the block
+        if (R32 + lane < rows) {
+            const int64_t tile = (R32 + lane) / g.rpt;
+            const int rr = (int)(R32 + lane - tile * g.rpt);
+            const int t0 = (int)(tile % g.nt[0]), t1 = (int)((tile / g.nt[0]) % g.nt[1]), t2 = (int)(tile / ((int64_t)g.nt[0] * g.nt[1]));
+            int c0, c1, c2;
+            row_coords(g.wide, rr, c0, c1, c2);
+            const int g0 = t0 * g.ts[0] + c0, g1 = t1 * g.ts[1] + c1, g2 = t2 * g.ts[2] + c2;
+            if (g0 < g.ext[0] && g1 < g.ext[1] && g2 < g.ext[2])
+                ro_mine = (int64_t)g0 * g.st[0] + (int64_t)g1 * g.st[1] + (int64_t)g2 * g.st[2];
+        }
+        const int64_t tile = R32 / g.rpt;                 // a tile has 64 or 128 rows: all 32 in one tile
+        const int rr32 = (int)(R32 - tile * g.rpt);
+        for (int it = 0; it < 4 * g.nch; ++it) {
+            const int ch = it >> 2, sub = (it & 3) * 8 + lane / 4;
+            const int64_t ro = __shfl_sync(0xffffffffu, ro_mine, sub);
+            float v[8];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {   // 16 summed indices (32 bytes per plane) at a time
-                uint32_t w[3][8];
+            for (int j = 0; j < 8; ++j) {
+                const int k = ch * tc::KCH + q * 8 + j;
+                const float *src = x + ro + (int64_t)k * g.sd;
+                v[j] = ro >= 0 && k < g.ed && dbg_ok(xr, src, 4, a.status) ? *src : 0.0f;
+            }
+            uint32_t w[3][4];
 #pragma unroll
-                for (int j = 0; j < 16; j += 2) {
-                    const int k = ch * tc::KCH + half * 16 + j;
-                    const float v0 = (valid && k < g.ed && dbg_ok(xr, x + ro + (int64_t)k * g.sd, 4, a.status))
-                                         ? x[ro + (int64_t)k * g.sd] : 0.0f;
-                    const float v1 = (valid && k + 1 < g.ed && dbg_ok(xr, x + ro + (int64_t)(k + 1) * g.sd, 4, a.status))
-                                         ? x[ro + (int64_t)(k + 1) * g.sd] : 0.0f;
-                    __nv_bfloat16 h0, m0, l0, h1, m1, l1;
-                    split_bf16x3(v0, h0, m0, l0);
-                    split_bf16x3(v1, h1, m1, l1);
-                    w[0][j >> 1] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-                    w[1][j >> 1] = (uint32_t)__bfloat16_as_ushort(m0) | ((uint32_t)__bfloat16_as_ushort(m1) << 16);
-                    w[2][j >> 1] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-                }
+            for (int j = 0; j < 4; ++j) {
+                __nv_bfloat16 h0, m0, l0, h1, m1, l1;
+                split_bf16x3(v[2 * j], h0, m0, l0);
+                split_bf16x3(v[2 * j + 1], h1, m1, l1);
+                w[0][j] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+                w[1][j] = (uint32_t)__bfloat16_as_ushort(m0) | ((uint32_t)__bfloat16_as_ushort(m1) << 16);
+                w[2][j] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+            }
 #pragma unroll
-                for (int pl = 0; pl < 3; ++pl) {
-                    uint4 *dst = base + (((tile * g.nch + ch) * 3 + pl) * g.rpt + rr) * 4 + half * 2;
-                    if (!dbg_ok(pr, dst, 32, a.status)) continue;
-                    dst[0] = make_uint4(w[pl][0], w[pl][1], w[pl][2], w[pl][3]);
-                    dst[1] = make_uint4(w[pl][4], w[pl][5], w[pl][6], w[pl][7]);
-                }
+            for (int pl = 0; pl < 3; ++pl) {
+                uint4 *dst = base + (((tile * g.nch + ch) * 3 + pl) * g.rpt + rr32 + sub) * 4 + q;
+                if (dbg_ok(pr, dst, 16, a.status)) *dst = make_uint4(w[pl][0], w[pl][1], w[pl][2], w[pl][3]);
             }
         }
     }
@@ -292,7 +306,7 @@ __global__ void __launch_bounds__(tc::THREADS, 1)
     uint64_t *full = bars, *empty = bars + RING, *tfull = bars + 2 * RING, *tempty = tfull + NACC, *mma_done = tempty + NACC;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    double *s_red = reinterpret_cast<double *>(tmem_slot + 4);     // DRAIN_WARPS partial sums
+    float2 *s_red = reinterpret_cast<float2 *>(tmem_slot + 4);     // DRAIN_WARPS partial sums and their errors
     int *s_geo = reinterpret_cast<int *>(s_red + DRAIN_WARPS);     // per term: pair-tile strides of
                                                                    // the wide labels 1, 2; narrow mask
     __shared__ float Tsh[TSZ];                                      // the pair-tile
@@ -431,6 +445,32 @@ __global__ void __launch_bounds__(tc::THREADS, 1)
             if (it != (int64_t)blockIdx.x) walk.next(a, t);
             const Item &item = walk.item;
             const int32_t *ext_b = a.ext + (int64_t)item.b * a.n_labels;
+            // the denominators of this thread's elements: it holds labels 0..3 at (et & 7, et >> 3 & 3,
+            // et >> 5 & 3, et >> 7) and labels 4, 5 at all 16 pairs.  Read before the terms, so that the
+            // loads (a pointer, then a value, per label) are over by the time the energy needs them.
+            const int c4[4] = {et & 7, (et >> 3) & 3, (et >> 5) & 3, (et >> 7) & 3};
+            bool v4 = true;
+            float d4 = 0.0f, ev[2][4];
+            int ok2[2];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int g = item.tc[q] * (q == 0 ? WA : TS) + c4[q];
+                const bool in = g < ext_b[a.t_col[q]];
+                v4 &= in;
+                if (in) d4 += a.sign[q] * reinterpret_cast<const float *>(a.eps[(int64_t)item.b * 6 + q])[g];
+            }
+#pragma unroll
+            for (int q = 4; q < 6; ++q) {
+                const float *eq = reinterpret_cast<const float *>(a.eps[(int64_t)item.b * 6 + q]);
+                ok2[q - 4] = 0;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int g = item.tc[q] * TS + c;
+                    const bool in = g < ext_b[a.t_col[q]];
+                    ok2[q - 4] |= (int)in << c;
+                    ev[q - 4][c] = in ? a.sign[q] * eq[g] : 0.0f;
+                }
+            }
             for (int p = 0; p < a.n_terms; ++p, ++tcount) {
                 const TermDev &tm = a.term[p];
                 const uint32_t ab = tcount % NACC, rnd = tcount / NACC;
@@ -461,57 +501,33 @@ __global__ void __launch_bounds__(tc::THREADS, 1)
                 }
                 named_bar_sync(1, 32 * DRAIN_WARPS);   // every term's additions before the next term's
             }
-            // energy of the pair-tile's elements inside the block: thread et holds labels 0..3 at
-            // (et & 7, et >> 3 & 3, et >> 5 & 3, et >> 7) and labels 4, 5 at all 16 pairs; D in
-            // FP32, T^2 / D summed in FP32 over the 16, then in FP64
-            double e_part = 0.0;
-            if (!dead) {
-                const int c4[4] = {et & 7, (et >> 3) & 3, (et >> 5) & 3, (et >> 7) & 3};
-                bool v4 = true;
-                float d4 = 0.0f;
+            // energy of the pair-tile's elements inside the block; T^2 / D summed in FP32 over the
+            // thread's 16 (j, k)
+            float hi = 0.0f, lo = 0.0f;
+            if (!dead && v4) {
+                const float *tp = Tsh + c4[0] + tstride(1) * c4[1] + tstride(2) * c4[2] + tstride(3) * c4[3];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int g = item.tc[q] * (q == 0 ? WA : TS) + c4[q];
-                    const bool in = g < ext_b[a.t_col[q]];
-                    v4 &= in;
-                    if (in) d4 += a.sign[q] * reinterpret_cast<const float *>(a.eps[(int64_t)item.b * 6 + q])[g];
-                }
-                if (v4) {
-                    float ev[2][4];
-                    int ok2[2];
-#pragma unroll
-                    for (int q = 4; q < 6; ++q) {
-                        const float *eq = reinterpret_cast<const float *>(a.eps[(int64_t)item.b * 6 + q]);
-                        ok2[q - 4] = 0;
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const int g = item.tc[q] * TS + c;
-                            const bool in = g < ext_b[a.t_col[q]];
-                            ok2[q - 4] |= (int)in << c;
-                            ev[q - 4][c] = in ? a.sign[q] * eq[g] : 0.0f;
-                        }
-                    }
-                    const float *tp = Tsh + c4[0] + tstride(1) * c4[1] + tstride(2) * c4[2] + tstride(3) * c4[3];
-                    float part = 0.0f;
-#pragma unroll
-                    for (int u = 0; u < 16; ++u) {
-                        const int cj = u & 3, ck = u >> 2;
-                        const bool in = ((ok2[0] >> cj) & 1) && ((ok2[1] >> ck) & 1);
-                        const float tv = tp[tstride(4) * cj + tstride(5) * ck];
-                        const float v = __fdividef(tv * tv, d4 + (ev[0][cj] + ev[1][ck]));
-                        part += in ? v : 0.0f;
-                    }
-                    e_part = (double)part;
+                for (int u = 0; u < 16; ++u) {
+                    const int cj = u & 3, ck = u >> 2;
+                    const bool in = ((ok2[0] >> cj) & 1) && ((ok2[1] >> ck) & 1);
+                    const float tv = tp[tstride(4) * cj + tstride(5) * ck];
+                    const float v = __fdividef(tv * tv, d4 + (ev[0][cj] + ev[1][ck]));
+                    hi += in ? v : 0.0f;
                 }
             }
+            // the 512 threads' sums with their exact rounding errors beside them: as accurate as FP64
+            // (2^-48), whose additions the SM does at two a clock (2560 of them a pair-tile took 4 % of it)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) e_part += __shfl_xor_sync(0xffffffffu, e_part, o);
-            if (lane == 0) s_red[warp - 2] = e_part;
+            for (int o = 16; o > 0; o >>= 1) add_exact(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
+            if (lane == 0) s_red[warp - 2] = make_float2(hi, lo);
             named_bar_sync(1, 32 * DRAIN_WARPS);   // the pair-tile is read; partial sums are in
-            if (et == 0) {
-                double sum = 0.0;
-                for (int w = 0; w < DRAIN_WARPS; ++w) sum += s_red[w];
-                if (sum != 0.0) atomicAdd(a.energies + item.b, sum);
+            if (warp == 2) {
+                const float2 v = s_red[lane & (DRAIN_WARPS - 1)];
+                hi = v.x;
+                lo = v.y;
+#pragma unroll
+                for (int o = DRAIN_WARPS / 2; o > 0; o >>= 1) add_exact(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
+                if (lane == 0 && hi != 0.0f) atomicAdd(a.energies + item.b, (double)hi + (double)lo);
             }
         }
     }
@@ -571,7 +587,9 @@ cudaError_t launch_triples_tc(const Plan &P, const Args &a, TcArgs t, cudaStream
         for (int b = t.b0; b < t.b1; ++b) batch_rows += tp.tc_rows[b];
         t.planes_bytes = batch_rows * tc::ROWB;
         const unsigned segs = (unsigned)((t.b1 - t.b0) * a.n_terms * 2);
-        triples_tc_split_kernel<<<segs, 256, 0, s>>>(a, t);
+        // about 16 CTAs per SM over the grid, at most 64 per operand
+        const unsigned shares = std::max(1u, std::min(64u, (152 * 16 + segs - 1) / segs));
+        triples_tc_split_kernel<<<dim3(segs, shares), 256, 0, s>>>(a, t);
         const int ctas = (int)std::min<int64_t>(t.n_items, std::max(1, sms));
         triples_tc_kernel<<<ctas, tc::THREADS, tc::SMEM, s>>>(map, a, t);
         cudaError_t e = cudaGetLastError();
