@@ -23,7 +23,7 @@
 //   warp 0       TMA producer: one 3-D tensor load per operand and stage brings both planes of
 //                the CTA's 128 rows of A and bn/2 rows of B, 64 K values, 128-byte swizzled; all
 //                of a stage's loads, from both CTAs, complete on CTA 0's barrier
-//   warp 1       allocates 512 tensor-memory columns (two accumulators); in CTA 0, lane 0 issues
+//   warp 1       allocates 512 tensor-memory columns (two accumulators); in CTA 0, one lane issues
 //                tcgen05.mma.cta_group::2 (M=256, N=bn, K=16) and commits to both CTAs
 //   warps 4..15  epilogue: each owns one tensor-memory lane quadrant and one third of the
 //                columns; drains an accumulator after every chunk into register sums (64 columns
@@ -31,8 +31,8 @@
 //                and at the end of the tile stores through the output's strides (the output
 //                permutation of TTGT folded in)
 //   3-stage shared-memory ring (56 KB per stage and CTA at bn = 192).
-// What bounds it: the power cap at large sizes.  M = N = K = 12288: 7.4-7.7 ms = 1.44-1.5 PFLOP/s of
-// MMA at 1630-1690 MHz (six bf16 products: 10.7-10.9 ms); ncu at 5120^3, alone: tensor pipe 93 %.
+// What bounds it: the power cap at large sizes.  M = N = K = 12288: 7.0 ms = 1.6 PFLOP/s of MMA
+// (six bf16 products: 10.7-10.9 ms); at middle sizes the hand-over of an accumulator per chunk (see NBUF).
 // Why pairs: with one CTA per 128 x 256 tile a stage reads 144 KB of operands from shared memory
 // and fills 96 KB per 1536 MMA cycles, 160 bytes per clock against the SM's 128; in a pair each
 // CTA holds half of B (bn = 192: 84 + 56 KB per 1152 cycles, 121).  Tiles of 240 and 256 columns run
@@ -63,10 +63,11 @@ constexpr int B_PLANE = BN / 2 * BK * 2;        // 12 KB at bn = 192
 constexpr int A_STAGE = 2 * A_PLANE;
 constexpr int STAGE_BYTES = A_STAGE + 2 * B_PLANE;   // 56 KB
 constexpr int EPI_WARPS = 12;                   // four lane quadrants x three column groups
-constexpr int GN = BN / 3;                      // columns per group (largest)
 constexpr int THREADS = 128 + 32 * EPI_WARPS;
-constexpr uint32_t TMEM_COLS = 512;             // two accumulators of 256 columns
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align*/ + BN * 8 /*c_col*/ + 256;
+constexpr uint32_t TMEM_COLS = 512;             // two accumulators of 256 columns, or eight of 64 (bn = 48)
+constexpr int MAXBUF = 8;
+constexpr int TURN = 32 * 17 * 4;               // one warp's 32 rows x 16 columns, turned (n_fast)
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align*/ + 2 * BN * 8 /*c_col*/ + 256 + EPI_WARPS * TURN;
 constexpr int STRIP = 24;                       // columns per block of the reduce kernel
 constexpr uint32_t SW128 = 2;                   // descriptor swizzle code: 128-byte swizzle
 constexpr uint32_t SBO = 8 * BK * 2;            // 8 rows of 128 bytes
@@ -74,6 +75,7 @@ constexpr uint32_t SBO = 8 * BK * 2;            // 8 rows of 128 bytes
 
 struct SplitArgs {
     uint32_t m_tiles, n_tiles;   // pair tiles
+    FastDiv fd_band, fd_last;    // division by 8 x n_tiles and by the last band's m-tiles
     uint32_t bn;                 // columns per pair tile
     uint32_t nch;                // K stages of 64
     uint32_t items;              // work items: m_tiles x n_tiles x ksplit
@@ -81,6 +83,7 @@ struct SplitArgs {
     uint32_t kslice_chunks;      // stages per slice
     uint32_t chunk_steps;        // K steps of 16 per accumulation chunk (4 or 2)
     uint32_t group;              // chunks per first-level sum
+    int n_fast;                  // C's stride-1 label is in the N group: a warp's stores run along columns
     float *partial;              // per slice, tile and CTA bn x 128 partial sums (scaled by
                                  // 2^(eA+eB)), [slice][tile][CTA][column][row], row fastest
     DbgRange dbg_p;              // debug builds: the partial sums' buffer
@@ -90,21 +93,32 @@ struct SplitArgs {
 };
 
 // work item's tile -> (m tile, n tile): bands of 8 m-tiles, n-major inside a band, for L2 reuse
-__device__ __forceinline__ void split_tile_coords(uint32_t tile, uint32_t m_tiles, uint32_t n_tiles, uint32_t &mt,
-                                                  uint32_t &nt) {
+__device__ __forceinline__ void split_tile_coords(uint32_t tile, const SplitArgs &x, uint32_t &mt, uint32_t &nt) {
     const uint32_t G = 8;
-    const uint32_t band = tile / (G * n_tiles);
+    const uint32_t band = fd_div(tile, x.fd_band);
     const uint32_t base = band * G;
-    const uint32_t g = min(G, m_tiles - base);
-    const uint32_t r = tile - band * G * n_tiles;
-    mt = base + r % g;
-    nt = r / g;
+    const uint32_t r = tile - band * G * x.n_tiles;
+    if (x.m_tiles - base >= G) {
+        mt = base + r % G;
+        nt = r / G;
+    } else {
+        nt = fd_div(r, x.fd_last);
+        mt = base + r - nt * (x.m_tiles - base);
+    }
+}
+
+// chunks of stages c0 .. c1 - 1: per_stage each, except that the end of K may leave the second half of its
+// stage empty
+__device__ __forceinline__ uint32_t split_chunk_count(uint32_t c0, uint32_t c1, uint32_t per_stage, uint32_t K) {
+    const uint32_t n = (c1 - c0) * per_stage;
+    return per_stage == 2 && c1 * split::BK >= K + split::BK / 2 ? n - 1 : n;
 }
 
 // The MMAs of one stage in chunks of STEPS K steps of 16 (32 bytes further in a swizzled row each),
-// corrections first; `ch` counts the chunks.  False: the wait for an accumulator ran out.
-template <int STEPS>
-__device__ __forceinline__ bool mma_stage(uint32_t sa, uint32_t sb, uint32_t b_plane, uint32_t idesc, uint32_t tmem,
+// corrections first, as far as k_steps steps hold K values; `ch` counts the chunks.  False: the wait for
+// an accumulator ran out.
+template <int STEPS, uint32_t nbuf>
+__device__ __forceinline__ bool mma_stage(int k_steps, uint32_t sa, uint32_t sb, uint32_t b_plane, uint32_t idesc, uint32_t tmem,
                                           uint32_t &ch, uint64_t *tfull, uint64_t *tempty, uint64_t tmo,
                                           volatile int *abort_flag) {
     using namespace split;
@@ -112,24 +126,29 @@ __device__ __forceinline__ bool mma_stage(uint32_t sa, uint32_t sb, uint32_t b_p
     const uint64_t ah = smem_desc(sa, 16, SBO, SW128), al = smem_desc(sa + A_PLANE, 16, SBO, SW128);
     const uint64_t bh = smem_desc(sb, 16, SBO, SW128), bl = smem_desc(sb + b_plane, 16, SBO, SW128);
 #pragma unroll
-    for (int k0 = 0; k0 < BK / 16; k0 += STEPS, ++ch) {
-        // accumulator ch % 2: the epilogue warps of both CTAs have drained it
-        const uint32_t buf = ch & 1, use = ch >> 1, acc = tmem + buf * 256;
-        if (use > 0 && !mbar_wait(&tempty[buf], (use - 1) & 1, tmo, abort_flag)) return false;
+    for (int k0 = 0; k0 < BK / 16; k0 += STEPS) {
+        if (k0 >= k_steps) break;
+        // accumulator ch % nbuf: the epilogue warps of both CTAs have drained it
+        const uint32_t buf = ch % nbuf, use = ch / nbuf, acc = tmem + buf * (nbuf == 3 ? 160 : 512 / nbuf);
+        if (use > 0 && !__all_sync(0xffffffffu, mbar_wait(&tempty[buf], (use - 1) & 1, tmo, abort_flag))) return false;
         tc_fence_after();
+        if (elect_one()) {
 #pragma unroll
-        for (int k = k0; k < k0 + STEPS; ++k) {
-            mma_f16_pair(acc, al + 2 * k, bh + 2 * k, idesc, k == k0 ? 0u : 1u);
-            mma_f16_pair(acc, ah + 2 * k, bl + 2 * k, idesc, 1);
+            for (int k = k0; k < k0 + STEPS; ++k) {
+                mma_f16_pair(acc, al + 2 * k, bh + 2 * k, idesc, k == k0 ? 0u : 1u);
+                mma_f16_pair(acc, ah + 2 * k, bl + 2 * k, idesc, 1);
+            }
+#pragma unroll
+            for (int k = k0; k < k0 + STEPS; ++k) mma_f16_pair(acc, ah + 2 * k, bh + 2 * k, idesc, 1);
+            mma_commit_pair(&tfull[buf]);   // chunk complete: ready to drain in both CTAs
         }
-#pragma unroll
-        for (int k = k0; k < k0 + STEPS; ++k) mma_f16_pair(acc, ah + 2 * k, bh + 2 * k, idesc, 1);
-        mma_commit_pair(&tfull[buf]);   // chunk complete: ready to drain in both CTAs
+        __syncwarp();
+        ++ch;
     }
     return true;
 }
 
-template <typename TOut, bool KSPLIT>
+template <typename TOut, bool KSPLIT, int NBUF>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
     gemm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                       const GemmParams p, const SplitArgs x) {
@@ -140,9 +159,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
     uint8_t *smem = smem_raw + (((raw + 1023) & ~1023u) - raw);
     uint8_t *stage_base = smem;
     int64_t *c_col = reinterpret_cast<int64_t *>(smem + STAGES * STAGE_BYTES);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + STAGES * STAGE_BYTES + BN * 8);
-    uint64_t *full = bars, *empty = bars + STAGES, *tfull = bars + 2 * STAGES, *tempty = tfull + 2,
-             *mma_done = tempty + 2;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + STAGES * STAGE_BYTES + 2 * BN * 8);
+    uint64_t *full = bars, *empty = bars + STAGES, *tfull = bars + 2 * STAGES, *tempty = tfull + MAXBUF,
+             *mma_done = tempty + MAXBUF;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
@@ -151,6 +170,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
     const uint32_t pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const uint64_t tmo = (uint64_t)p.timeout_ns;
     const uint32_t tiles = x.m_tiles * x.n_tiles;
+    // Accumulators: as many as tensor memory holds of the tile's columns (2 of 256, 3 of 160, 4 of 128).  With
+    // two, a chunk of 32 K values takes the round trip of a hand-over, about 1050 clocks, whatever
+    // its width.
+    // NBUF 8 (narrow tiles of few chunks): each group of four epilogue warps takes whole tiles in turn,
+    // three at a time, and tensor memory holds eight accumulators.  With a third of 48 columns per warp
+    // the fixed work per tile (offsets, waits, a barrier) was most of it: 995 K x 48, K = 48: 177 us,
+    // 130 us so.  A tile has at most three chunks then: a group that has seen its last tile's chunks
+    // waits for one at most seven further on, so the accumulator's phase before that one is over and the
+    // parity it waits for is not the older phase's.
+    constexpr bool solo = NBUF == 8;
+    constexpr uint32_t nbuf = NBUF, buf_cols = NBUF == 3 ? 160 : 512 / NBUF;
+    constexpr int GN = NBUF == 2 ? 64 : NBUF == 4 ? 32 : 48;   // a warp's columns, at most
     const uint32_t stage_bytes = (uint32_t)A_STAGE + x.bn * (BK * 2);   // one CTA's loads of a stage
     // work item t: K slice t / tiles of output tile t % tiles
     auto kslice = [&](uint32_t t, uint32_t &c0, uint32_t &c1) -> uint32_t {
@@ -168,7 +199,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&tfull[b], 1); mbar_init(&tempty[b], 2 * EPI_WARPS); }
+        for (int b = 0; b < MAXBUF; ++b) { mbar_init(&tfull[b], 1); mbar_init(&tempty[b], 2 * (solo ? 4 : EPI_WARPS)); }
         mbar_init(mma_done, 1);
         *abort_flag = 0;
         fence_barrier_init();
@@ -189,7 +220,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
     };
     auto tile_coords = [&](uint32_t t, uint32_t &mt, uint32_t &nt) {
         if constexpr (KSPLIT) t %= tiles;
-        split_tile_coords(t, x.m_tiles, x.n_tiles, mt, nt);
+        split_tile_coords(t, x, mt, nt);
     };
 
     // registers: 512 threads launch at 128 each; 12 x 32 x 160 + 4 x 32 x 32 = 65536
@@ -231,8 +262,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
             }
         }
     } else if (warp == 1) {
-        if (rank == 0 && lane == 0) {
-            // ---------------- MMA issuer ----------------
+        if (rank == 0) {
+            // ---------------- MMA issuer (the whole warp; one lane issues) ----------------
             const uint32_t idesc = idesc_f16_f32(2 * BM, x.bn);
             const uint32_t b_plane = x.bn / 2 * (BK * 2);
             uint32_t it = 0, ch = 0;   // stages and chunks so far
@@ -242,16 +273,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
                 kslice(t, c0, c1);
                 for (uint32_t c = c0; c < c1; ++c, ++it) {
                     const uint32_t s = it % STAGES, round = it / STAGES;
-                    if (!mbar_wait(&full[s], round & 1, tmo, abort_flag)) { fail(); ok = false; break; }
+                    ok = __all_sync(0xffffffffu, mbar_wait(&full[s], round & 1, tmo, abort_flag));
+                    if (!ok) { if (lane == 0) fail(); break; }
                     const uint32_t sa = smem_u32(stage_base + s * STAGE_BYTES), sb = sa + A_STAGE;
-                    ok = x.chunk_steps == 4 ? mma_stage<4>(sa, sb, b_plane, idesc, tmem_base, ch, tfull, tempty, tmo, abort_flag)
-                                            : mma_stage<2>(sa, sb, b_plane, idesc, tmem_base, ch, tfull, tempty, tmo, abort_flag);
-                    if (!ok) { fail(); break; }
-                    mma_commit_pair(&empty[s]);   // the stage is free in both CTAs once read
+                    const int k_steps = (int)(min(p.K - c * BK, (uint32_t)BK) + 15) / 16;
+                    ok = x.chunk_steps == 4 ? mma_stage<4, nbuf>(k_steps, sa, sb, b_plane, idesc, tmem_base, ch, tfull, tempty, tmo, abort_flag)
+                                            : mma_stage<2, nbuf>(k_steps, sa, sb, b_plane, idesc, tmem_base, ch, tfull, tempty, tmo, abort_flag);
+                    if (!ok) { if (lane == 0) fail(); break; }
+                    if (elect_one()) mma_commit_pair(&empty[s]);   // the stage is free in both CTAs once read
+                    __syncwarp();
                 }
             }
             // make sure no MMA is still writing tensor memory before it is freed
-            mma_commit_pair(mma_done);
+            if (elect_one()) mma_commit_pair(mma_done);
+            __syncwarp();
             mbar_wait(mma_done, 0, tmo, nullptr);
         }
     }
@@ -259,54 +294,89 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
         regs_up<160>();
         // ---------------- epilogue (warps 4..15) ----------------
         const int quad = warp & 3;                  // tensor-memory lanes 32*quad .. 32*quad+31
-        const uint32_t gn = x.bn / 3, g0 = (uint32_t)((warp - 4) >> 2) * gn;   // columns g0 .. g0 + gn - 1
-        const int et = threadIdx.x - 128;           // 0..383
+        const uint32_t grp = (uint32_t)(warp - 4) >> 2;
+        const uint32_t gn = solo ? x.bn : x.bn / 3, g0 = solo ? 0 : grp * gn;   // columns g0 .. g0 + gn - 1
+        const int meet = solo ? 128 : 32 * EPI_WARPS;                          // threads that share a tile
+        const int et = solo ? (int)(threadIdx.x & 127) : (int)threadIdx.x - 128;
+        int64_t *cols = c_col + (solo ? grp * 128 : 0);                        // two tiles' column offsets
+        const uint32_t cols_half = solo ? 64 : BN;
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
         const int e_sum = half_exponent<TOut>(scale_exponent<TOut>(x.scale_a)) +
                           half_exponent<TOut>(scale_exponent<TOut>(x.scale_b));
         // 2^(eA+eB-28) in two factors: the sums carry 2^28 more than the result's scale
         constexpr float kShift = 1.0f / (float)(1 << (2 * kHalfShift));
         const uint32_t tempty0 = map_to_rank(tempty, 0);
+        const double scale = ldexp(p.alpha, e_sum);
+        const TOut sc = (TOut)scale;
+        const bool plain = p.beta == 0.0;
+        float *turn = reinterpret_cast<float *>(smem + STAGES * STAGE_BYTES + 2 * BN * 8 + 256) + (warp - 4) * (TURN / 4);
         uint32_t ch = 0;     // chunks so far
+        uint32_t cb = 0;     // this tile's half of c_col
         const uint32_t per_stage = BK / 16 / x.chunk_steps;
         bool dead = false;   // once set, the warp keeps pace with the barriers but does no work
         TOut *C = reinterpret_cast<TOut *>(p.C);
+        uint32_t turn_of = 0;   // the group whose turn the item is (narrow tiles)
         for (uint32_t t = pair; t < x.items; t += n_pairs) {
             uint32_t mt, nt, c0, c1;
-            tile_coords(t, mt, nt);
             const uint32_t ks = kslice(t, c0, c1);
+            const uint32_t n_ch = split_chunk_count(c0, c1, per_stage, p.K);
+            const bool mine = !solo || turn_of == grp;
+            turn_of = turn_of == 2 ? 0 : turn_of + 1;
+            if (!mine) {
+                ch += n_ch;
+                continue;
+            }
+            tile_coords(t, mt, nt);
+            int64_t c_row = 0;
             if constexpr (!KSPLIT) {
-                // column offsets of this tile in C (all eight epilogue warps always meet here)
-                named_bar_sync(1, 32 * EPI_WARPS);
+                // offsets of this tile's columns in C, in the half that no warp still reads (all
+                // epilogue warps meet here, so the half's last readers are two tiles back), and of
+                // this thread's row
+                cb ^= 1;
                 int64_t o0 = 0, o1 = 0;
                 if ((uint32_t)et < x.bn && nt * x.bn + et < p.N) radix_offsets(p.nb, nt * x.bn + et, o0, o1);
-                if (et < BN) c_col[et] = o1;
-                named_bar_sync(1, 32 * EPI_WARPS);
+                if (et < (int)cols_half) cols[cb * cols_half + et] = o1;
+                const uint32_t mr = mt * (2 * BM) + rank * BM + quad * 32 + lane;
+                if (mr < p.M) radix_offsets(p.ma, mr, o0, c_row);
+                named_bar_sync(solo ? 1 + (int)grp : 1, meet);   // ids 1..3
             }
             // two levels of sums, two columns per register pair: T over x.group chunks, S over the groups
             uint64_t T[GN / 2], S[GN / 2];
 #pragma unroll
-            for (int j = 0; j < GN / 2; ++j) T[j] = S[j] = 0;
-            const uint32_t n_ch = (c1 - c0) * per_stage;
+            for (int c16 = 0; c16 < GN / 16; ++c16)   // a narrow tile works on the columns that it has
+                if ((uint32_t)c16 * 16 < gn) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) T[c16 * 8 + q] = S[c16 * 8 + q] = 0;
+                }
             uint32_t left = x.group;
             for (uint32_t c = 0; c < n_ch; ++c, ++ch) {
                 if (dead) continue;
-                const uint32_t buf = ch & 1;
-                bool ok = mbar_wait(&tfull[buf], (ch >> 1) & 1, tmo, abort_flag);
+                const uint32_t buf = ch % nbuf;
+                bool ok = mbar_wait(&tfull[buf], (ch / nbuf) & 1, tmo, abort_flag);
                 ok = __all_sync(0xffffffffu, ok);   // warp-uniform before the .sync.aligned loads
                 if (!ok) { if (lane == 0) fail(); dead = true; continue; }
                 tc_fence_after();
-                const uint32_t src = tmem_base + lane_base + buf * 256 + g0;
+                const uint32_t src = tmem_base + lane_base + buf * buf_cols + g0;
+                if constexpr (GN == 32) {   // both loads, then one wait: the registers allow it here
+                    uint32_t r[32];
+                    tmem_ld16(src, *reinterpret_cast<uint32_t(*)[16]>(&r[0]));
+                    if (gn > 16) tmem_ld16(src + 16, *reinterpret_cast<uint32_t(*)[16]>(&r[16]));
+                    tmem_ld_wait();
 #pragma unroll
-                for (int c16 = 0; c16 < GN / 16; ++c16) {
-                    if ((uint32_t)c16 * 16 < gn) {
-                        uint32_t r[16];
-                        tmem_ld16(src + c16 * 16, r);
-                        tmem_ld_wait();
+                    for (int q = 0; q < 16; ++q)
+                        if (q < 8 || gn > 16) T[q] = f32x2_add(T[q], f32x2_pack(r[2 * q], r[2 * q + 1]));
+                } else {
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            uint64_t &t = T[c16 * 8 + q];
-                            t = f32x2_add(t, f32x2_pack(r[2 * q], r[2 * q + 1]));
+                    for (int c16 = 0; c16 < GN / 16; ++c16) {
+                        if ((uint32_t)c16 * 16 < gn) {
+                            uint32_t r[16];
+                            tmem_ld16(src + c16 * 16, r);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                uint64_t &t = T[c16 * 8 + q];
+                                t = f32x2_add(t, f32x2_pack(r[2 * q], r[2 * q + 1]));
+                            }
                         }
                     }
                 }
@@ -316,10 +386,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
                 if (--left == 0 || c + 1 == n_ch) {
                     left = x.group;
 #pragma unroll
-                    for (int j = 0; j < GN / 2; ++j) {
-                        S[j] = f32x2_add(S[j], T[j]);
-                        T[j] = 0;
-                    }
+                    for (int c16 = 0; c16 < GN / 16; ++c16)
+                        if ((uint32_t)c16 * 16 < gn) {
+#pragma unroll
+                            for (int j = c16 * 8; j < c16 * 8 + 8; ++j) {
+                                S[j] = f32x2_add(S[j], T[j]);
+                                T[j] = 0;
+                            }
+                        }
                 }
             }
             if (dead) continue;
@@ -332,25 +406,58 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
             const int n_here = (int)min(gn, p.N > n0 ? p.N - n0 : 0u);
             if constexpr (KSPLIT) {   // K slice partial: scaled sums to the tile's slot, row fastest (coalesced)
                 if (m < p.M) {
-                    const float sc = (float)ldexp(1.0, e_sum);
+                    const float sp = (float)ldexp(1.0, e_sum);
                     float *P = x.partial + ((((size_t)ks * tiles + t % tiles) * 2 + rank) * x.bn + g0) * BM + ml;
 #pragma unroll
                     for (int j = 0; j < GN; ++j)
                         if (j < n_here && dbg_ok(x.dbg_p, P + (size_t)j * BM, 4, p.status))
-                            P[(size_t)j * BM] = sc * result(j);
+                            P[(size_t)j * BM] = sp * result(j);
+                }
+            } else if (x.n_fast) {
+                // through shared memory, 16 columns at a time, so that sixteen lanes store one row's
+                // columns (64-byte runs): along the rows each store would touch 32 sectors
+                                const int64_t *cc = cols + cb * cols_half + g0;
+                const int m_here = (int)min(32u, p.M > m - lane ? p.M - (m - lane) : 0u);   // the warp's rows inside C
+#pragma unroll
+                for (int c16 = 0; c16 < GN / 16; ++c16) {
+                    if (c16 * 16 < n_here) {   // uniform over the warp
+                        __syncwarp();
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) turn[lane * 17 + j] = result(c16 * 16 + j);
+                        __syncwarp();
+                        const int col = lane & 15;
+                        const bool in_n = c16 * 16 + col < n_here;
+                        TOut *at = C + cc[c16 * 16 + col];
+                        // two loops: FP64 conversions on the += path must not be computed for the plain one
+                        if (plain) {
+#pragma unroll 4
+                            for (int r = lane >> 4; r < 32; r += 2) {
+                                TOut *dst = at + __shfl_sync(0xffffffffu, c_row, r);
+                                if (r < m_here && in_n && dbg_ok(p.dbg_c, dst, (int)sizeof(TOut), p.status))
+                                    *dst = sc * (TOut)turn[r * 17 + col];
+                            }
+                        } else {
+#pragma unroll 1
+                            for (int r = lane >> 4; r < 32; r += 2) {
+                                TOut *dst = at + __shfl_sync(0xffffffffu, c_row, r);
+                                if (r < m_here && in_n && dbg_ok(p.dbg_c, dst, (int)sizeof(TOut), p.status))
+                                    *dst = (TOut)(scale * (double)turn[r * 17 + col] + p.beta * (double)*dst);
+                            }
+                        }
+                    }
                 }
             } else if (m < p.M) {
-                int64_t r0 = 0, c_row = 0;
-                radix_offsets(p.ma, m, r0, c_row);
                 TOut *row = C + c_row;
-                const int64_t *cc = c_col + g0;
-                const double scale = ldexp(p.alpha, e_sum);
-                if (p.beta == 0.0) {
-                    const TOut sc = (TOut)scale;
+                const int64_t *cc = cols + cb * cols_half + g0;
+                if (plain) {
 #pragma unroll
-                    for (int j = 0; j < GN; ++j)
-                        if (j < n_here && dbg_ok(p.dbg_c, row + cc[j], (int)sizeof(TOut), p.status))
-                            row[cc[j]] = sc * (TOut)result(j);
+                    for (int c16 = 0; c16 < GN / 16; ++c16)
+                        if (c16 * 16 < n_here) {
+#pragma unroll
+                            for (int j = c16 * 16; j < c16 * 16 + 16; ++j)
+                                if (j < n_here && dbg_ok(p.dbg_c, row + cc[j], (int)sizeof(TOut), p.status))
+                                    row[cc[j]] = sc * (TOut)result(j);
+                        }
                 } else {
 #pragma unroll
                     for (int j = 0; j < GN; ++j)
@@ -382,7 +489,7 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmParams p, c
     const uint32_t strips = x.bn / STRIP;
     const uint32_t strip = blockIdx.x % strips, cta = blockIdx.x / strips, tile = cta >> 1, rank = cta & 1;
     uint32_t mt, nt;
-    split_tile_coords(tile, x.m_tiles, x.n_tiles, mt, nt);
+    split_tile_coords(tile, x, mt, nt);
     const uint32_t ml = threadIdx.x & 127, m = mt * (2 * BM) + rank * BM + ml, n0 = nt * x.bn + strip * STRIP;
     if (threadIdx.x < STRIP && n0 + threadIdx.x < p.N) {
         int64_t o0, o1;
@@ -463,16 +570,16 @@ static int sm_count() {
 }
 
 // the shared-memory attribute is set once per kernel instantiation
-template <typename TOut, bool KSPLIT>
+template <typename TOut, bool KSPLIT, int NBUF>
 static void launch_split_kernel(const CUtensorMap &ta, const CUtensorMap &tb, const GemmParams &p,
                                 const SplitArgs &x, int ctas, cudaStream_t s) {
     static const bool attr = [] {
-        cudaFuncSetAttribute(gemm_split_kernel<TOut, KSPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(gemm_split_kernel<TOut, KSPLIT, NBUF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              split::SMEM_BYTES);
         return true;
     }();
     (void)attr;
-    launch_pdl(gemm_split_kernel<TOut, KSPLIT>, ctas, split::THREADS, split::SMEM_BYTES, s, ta, tb, p, x);
+    launch_pdl(gemm_split_kernel<TOut, KSPLIT, NBUF>, ctas, split::THREADS, split::SMEM_BYTES, s, ta, tb, p, x);
 }
 
 cudaError_t launch_gemm_split(const GemmParams &p, const void *parts_a, const void *parts_b,
@@ -489,6 +596,8 @@ cudaError_t launch_gemm_split(const GemmParams &p, const void *parts_a, const vo
     SplitArgs x;
     x.m_tiles = (p.M + kSplitBM - 1) / kSplitBM;
     x.n_tiles = (p.N + sch.bn - 1) / sch.bn;
+    x.fd_band = make_fastdiv(8 * x.n_tiles);
+    x.fd_last = make_fastdiv(x.m_tiles % 8 ? x.m_tiles % 8 : 8);
     x.bn = sch.bn;
     x.nch = (p.K + BK - 1) / BK;
     x.ksplit = sch.ksplit;
@@ -497,17 +606,25 @@ cudaError_t launch_gemm_split(const GemmParams &p, const void *parts_a, const vo
     split_chunks(x.kslice_chunks, &x.chunk_steps, &x.group);
     x.partial = partial;
     x.dbg_p = dbg_range(partial, split_partial_bytes(p.M, p.N, sch));
+    // along columns where the N group's first label is C's stride-1 label (and the M group's is not)
+    x.n_fast = p.nb.n > 0 && p.nb.s1[0] == 1 && p.nb.ext[0] > 1 && !(p.ma.n > 0 && p.ma.s1[0] == 1 && p.ma.ext[0] > 1);
     x.debug_flags = debug_flags;
     x.scale_a = scale_a;
     x.scale_b = scale_b;
     const int ctas = 2 * (int)std::min(pairs, x.items);
-    if (out_bytes == 8) {
-        if (x.ksplit > 1) launch_split_kernel<double, true>(ta, tb, p, x, ctas, s);
-        else launch_split_kernel<double, false>(ta, tb, p, x, ctas, s);
-    } else {
-        if (x.ksplit > 1) launch_split_kernel<float, true>(ta, tb, p, x, ctas, s);
-        else launch_split_kernel<float, false>(ta, tb, p, x, ctas, s);
-    }
+    const bool solo = x.bn == 48 && x.ksplit == 1 && split_chunks_of(x.nch, x.chunk_steps, p.K) <= 3;
+    const int nbuf = solo ? 8 : x.bn <= 128 ? 4 : x.bn <= 160 ? 3 : 2;
+#define CM_SPLIT(T, K, B) launch_split_kernel<T, K, B>(ta, tb, p, x, ctas, s)
+#define CM_SPLIT_T(T)                                                                   \
+    do {                                                                                \
+        if (x.ksplit > 1) nbuf == 4 ? CM_SPLIT(T, true, 4) : nbuf == 3 ? CM_SPLIT(T, true, 3) : CM_SPLIT(T, true, 2); \
+        else if (solo) CM_SPLIT(T, false, 8);                                           \
+        else nbuf == 4 ? CM_SPLIT(T, false, 4) : nbuf == 3 ? CM_SPLIT(T, false, 3) : CM_SPLIT(T, false, 2); \
+    } while (0)
+    if (out_bytes == 8) CM_SPLIT_T(double);
+    else CM_SPLIT_T(float);
+#undef CM_SPLIT_T
+#undef CM_SPLIT
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || x.ksplit == 1) return e;
     const uint32_t blocks = x.m_tiles * x.n_tiles * 2 * (x.bn / STRIP);

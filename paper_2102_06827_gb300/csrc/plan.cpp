@@ -409,6 +409,8 @@ void cost_form(const Plan &P, const std::vector<int> &lx, const std::vector<int>
     auto sz = label_strides(zl, ext);
     double run_c = (double)contiguous_run(f->M, sz, ext);
     f->eff_store = run_eff(std::min(run_c, 32.0) * es * 2);
+    if (kernel == KK_GEMM_SPLIT)   // its epilogue turns tiles whose columns are the result's runs
+        f->eff_store = std::max(f->eff_store, 0.8 * run_eff(std::min((double)contiguous_run(f->N, sz, ext), 16.0) * es));
     double t_store = M * N * es / (kHbmBytesPerS * f->eff_store);
     if (kernel == KK_GEMM_SPLIT || kernel == KK_GEMM_EMU) {
         // pre-passes: read the operand, write 2 FP16 (split) or 6 bf16 (emulated FP64) planes in
@@ -1082,7 +1084,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             st.ksplit = sch.ksplit;
             st.tile_n = sch.bn;
             // one launch on the FP32 pipes where that is modelled faster than the split form's chain
-            // (about 9 us of pre-passes and launches around its GEMM); asking for K slices or for the
+            // (about 8 us of pre-passes and launches around its GEMM); asking for K slices or for the
             // fault injection keeps the split form
             const Slot &sm = P->slots[st.form.swap ? st.b : st.a], &sn = P->slots[st.form.swap ? st.a : st.b];
             auto run = [&](const Slot &s, const std::vector<int> &rows) {
@@ -1091,7 +1093,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             };
             const bool long_runs = run(sm, st.form.M) >= 16 && run(sn, st.form.N) >= 16;
             st.small = P->dtype == COMET_F32 && opts.ksplit <= 0 && !(opts.debug_flags & 1) &&
-                       small_gemm_us((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, long_runs) < sch.us + 9.0;
+                       small_gemm_us((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, long_runs) < sch.us + 8.0;
             bk = (size_t)split_partial_bytes((uint64_t)rows_a, (uint64_t)rows_b, sch);
             const int64_t tiles = ((rows_a + 127) / 128) * ((rows_b + 255) / 256), tail = tiles % 152;
             st.tail_tiles = 0;

@@ -18,6 +18,16 @@ __device__ __forceinline__ uint64_t globaltimer() {
     return t;
 }
 
+// True in one lane of the (converged) warp.  Tensor-core instructions take their operands from
+// uniform registers: a loop that the whole warp runs, with only the instruction itself under this
+// predicate, keeps descriptors and addresses there, where code under `lane == 0` has to move each of
+// them over for every instruction (about 130 clocks per MMA in the split GEMM).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.b32 %0, 1, 0, q;\n\t}\n" : "=r"(p));
+    return p != 0;
+}
+
 // ---- mbarrier -------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");

@@ -37,31 +37,43 @@ inline int64_t split_partial_bytes(uint64_t M, uint64_t N, const SplitSchedule &
     return tiles * s.ksplit * kSplitBM * s.bn * 4;
 }
 
+// Chunks of a whole-K tile: the end of K may leave the second half of its stage empty.
+inline uint32_t split_chunks_of(uint32_t stages, uint32_t steps, uint64_t K) {
+    const uint32_t n = stages * (4 / steps);
+    return steps == 2 && (uint64_t)stages * kSplitBK >= K + kSplitBK / 2 ? n - 1 : n;
+}
+
 // The schedule with the least modelled time over the tile widths and K slices whose partial
 // sums fit `partial_limit` bytes.  want_ksplit: 0 = free, k = as near to k slices as K allows.
-// The model, at 1.9 GHz: a pair's stage of 64 K values takes 6 * bn cycles of MMA, but not less
-// than 1000 (its loads: (128 + bn/2) * 256 bytes per SM at what the L2 gives all SMs together); a tile
-// takes 5000 + 10 * bn cycles around its main loop (pipeline fill, last drain, stores); K slices
-// add a launch and their partial sums' traffic.
+// The model, in clocks at 1.9 GHz, from kernel times on 1633^3, 2700^3, 4864 x 960 x 4800, 200000 x 48 x
+// (96, 160) and 200000 x 192 x 48 at every width: a stage of 64 K values takes 1300 / 1420 / 1860 / 2150
+// (widths 48 / 96 / 144 / 192) in chunks of 32 and 1000 / 1130 / 1320 / 1480 in chunks of 64, a tile 2000 +
+// 26 a column around its stages, or 4700 in all for a narrow tile of at most three chunks; 3000 once; K
+// slices add a launch and their partial sums' traffic.
 inline SplitSchedule split_schedule(uint64_t M, uint64_t N, uint64_t K, uint32_t pairs, uint32_t want_ksplit,
                                     int64_t partial_limit) {
+    static const double stage32[4] = {1300, 1420, 1860, 2150}, stage64[4] = {1000, 1130, 1320, 1480};
     const uint64_t mt = (M + kSplitBM - 1) / kSplitBM;
     const uint32_t nch = (uint32_t)std::max<uint64_t>(1, (K + kSplitBK - 1) / kSplitBK);
     SplitSchedule best;
     bool have = false;
-    for (uint32_t bn = 48; bn <= (uint32_t)kSplitMaxBN; bn += 48) {
+    for (uint32_t w = 0; w < 4; ++w) {
+        const uint32_t bn = 48 * (w + 1);
         const uint64_t tiles = mt * ((N + bn - 1) / bn);
-        const double chunk = std::max(6.0 * bn, std::max(1000.0, (128 + bn / 2) * 256 / 48.0));
         const uint32_t k_lo = want_ksplit ? std::min(want_ksplit, nch) : 1, k_hi = want_ksplit ? k_lo : std::min(16u, nch);
         for (uint32_t k = k_lo; k <= k_hi; ++k) {
             SplitSchedule s;
             const uint32_t per = (nch + k - 1) / k;
             s.bn = bn;
-            s.ksplit = (nch + per - 1) / per;   // every slice holds at least one chunk
+            s.ksplit = (nch + per - 1) / per;   // every slice holds at least one stage
             const int64_t pb = split_partial_bytes(M, N, s);
             if (pb > partial_limit) continue;
+            uint32_t steps, group;
+            split_chunks(per, &steps, &group);
             const double waves = (double)((tiles * s.ksplit + pairs - 1) / pairs);
-            s.us = waves * (per * chunk + 5000 + 10.0 * bn) / 1900.0;
+            const bool narrow = w == 0 && s.ksplit == 1 && split_chunks_of(nch, steps, K) <= 3;
+            const double tile = narrow ? 4700.0 : per * (steps == 2 ? stage32 : stage64)[w] + 2000.0 + 26.0 * bn;
+            s.us = (3000.0 + waves * tile) / 1900.0;
             if (s.ksplit > 1) s.us += 3.0 + (double)pb / 2.0e6;   // written and read back, mostly in L2
             if (!have || s.us < best.us * (1 - 1e-9)) { best = s; have = true; }
         }

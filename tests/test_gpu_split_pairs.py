@@ -74,3 +74,25 @@ def test_scale_slots_ignore_non_finite_elements(comet, M, N, K, views):
     fine[[3, M - 1]] = False
     assert normwise(C[fine], ref[fine]) <= 6e-7
     assert not np.isfinite(C[~fine]).any()
+
+
+@pytest.mark.parametrize("expr", [E, "C[n,m] = A[k,m] * B[k,n]"])
+@pytest.mark.parametrize("M,N,K", [(128 * 400 + 1, 48, 48), (128 * 400 + 1, 47, 96), (128 * 400 - 1, 48, 97),
+                                   (128 * 400, 33, 128), (100, 3001, 96), (257, 191, 1000)])
+def test_narrow_tiles_and_either_direction_of_the_result(comet, expr, M, N, K):
+    # one group per tile up to 96 values of K and three groups above, rows of the result along M and along
+    # N (odd extents: unaligned runs), stored and accumulated
+    ext = dict(m=M, n=N, k=K)
+    lhs = [M, N] if expr is E else [N, M]
+    A, B = f32((K, M), 75, 0, kind="normal"), f32((K, N), 75, 1, kind="normal")
+    ref = oracle.einsum(expr, A, B)
+    import torch
+    for scale in ("", "1.5 * ", "+"):
+        e = expr.replace("= ", "+= 0.5 * ") if scale == "+" else expr.replace("= ", "= " + scale)
+        p = comet.Plan(e, ext, torch.float32, precision="split_bf16", ksplit=1)
+        C0 = f32(lhs, 75, 2, kind="normal")
+        out = to_dev(C0, np.float32)
+        p.contract([to_dev(a, np.float32) for a in (A, B)], out, p.workspace())
+        comet.sync_status()
+        want = C0 + 0.5 * ref if scale == "+" else (1.5 if scale else 1.0) * ref
+        assert normwise(from_dev(out).astype(np.float64), want) <= 6e-7
