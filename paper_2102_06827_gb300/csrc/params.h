@@ -160,8 +160,12 @@ struct GemvParams {
     void *Y;
     double alpha, beta;
     int n_fast;                    // 1: X's stride-1 dim is a free digit, 0: a contracted one
+    int vec4;                      // X can be read four elements at a time along its stride-1 digit: that
+                                   // digit comes first, its extent and every other X stride are
+                                   // multiples of four (X itself 16-byte aligned: checked at launch)
     int v_ones;                    // 1: v is all ones (a sum over the k digits of X; v unused)
-    uint32_t nchunks;              // ceil(K / 1024)
+    uint32_t kc;                   // k values per chunk (gemv_chunk): a multiple of 128, at most 1024
+    uint32_t nchunks;              // ceil(K / kc)
     double *partial;               // workspace: n_batch x nchunks x N FP64 partial sums
     DbgRange dbg_v, dbg_x, dbg_y, dbg_p;   // debug builds: the buffers of v, X, Y and partial
     int *status;                   // debug builds: device status word

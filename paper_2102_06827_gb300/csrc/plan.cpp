@@ -492,6 +492,31 @@ void prepass_params(const Step &st, const std::vector<int> &labels, std::map<int
     xp->out_plane = prod_ext(ext, rows) * st.kpad;
 }
 
+// Whether a gemv step's X can be read in vectors of four elements (GemvParams::vec4)
+int gemv_vec4(const GemvParams &v) {
+    const Radix &f = v.n_fast ? v.n : v.k, &o = v.n_fast ? v.k : v.n;
+    const int64_t *fs = v.n_fast ? f.s0 : f.s1, *os = v.n_fast ? o.s1 : o.s0;
+    if (f.n == 0 || fs[0] != 1 || f.ext[0] % 4) return 0;
+    for (int d = 1; d < f.n; ++d) if (fs[d] % 4) return 0;
+    for (int d = 0; d < o.n; ++d) if (os[d] % 4) return 0;
+    for (int d = 0; d < v.bv.n; ++d) if (v.bv.s1[d] % 4) return 0;
+    return 1;
+}
+
+// Values of K per block of a gemv step: 1024, halved down to 128 while the grid leaves the 152 SMs with
+// fewer than four blocks each (at 1024 a 1.7 M element operand made 28 blocks and took 40 us, now
+// 14 us; from four blocks on an SM shorter chunks only add partial sums).  `base` is where the
+// partial sums start in the workspace: they never grow past 31 MiB, so that a plan that fits the
+// no-alloc scratch with whole chunks still does.
+uint32_t gemv_chunk(int64_t N, int64_t K, int64_t n_batch, int n_fast, size_t base) {
+    const int64_t tiles = n_batch * ((N + (n_fast ? 127 : 63)) / (n_fast ? 128 : 64));
+    int64_t kc = 1024;
+    while (kc > 128 && K > kc / 2 && tiles * ((K + kc - 1) / kc) < 4 * 152 && (K + kc / 2 - 1) / (kc / 2) <= 65535 &&
+           base + (size_t)(n_batch * N * ((K + kc / 2 - 1) / (kc / 2)) * 8) <= (31u << 20))
+        kc /= 2;
+    return (uint32_t)kc;
+}
+
 // Slices of the host-buffer pipeline (see HostPipe).  The slicing minimises a small event
 // model: the inputs cross the host link one after another in the copy order, each slice's
 // pre-pass runs before its first GEMM block, a block starts when its slices are pre-passed and
@@ -1131,11 +1156,13 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             for (int d = 0; d < v.n.n; ++d) min_n = std::min(min_n, v.n.s0[d]);
             for (int d = 0; d < v.k.n; ++d) min_k = std::min(min_k, v.k.s1[d]);
             v.n_fast = min_n < min_k ? 1 : 0;
-            v.nchunks = (v.K + 1023) / 1024;
+            v.kc = gemv_chunk(v.N, v.K, 1, v.n_fast, parts_base);
+            v.nchunks = (v.K + v.kc - 1) / v.kc;
             v.v_ones = 1;
             v.n_batch = 1;
             v.bv.total = 1;
             v.by.total = 1;
+            v.vec4 = gemv_vec4(v);
             st.ws_partial = parts_base;
             parts_max = std::max(parts_max, align((size_t)v.nchunks * (size_t)v.N * 8));
             continue;
@@ -1144,7 +1171,12 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
         const int64_t Kx = prod_ext(P->extent, st.form.K);
         const int64_t Nx = prod_ext(P->extent, st.form.M.empty() ? st.form.N : st.form.M);
         st.ws_partial = parts_base;
-        parts_max = std::max(parts_max, align((size_t)st.n_batch * (size_t)((Kx + 1023) / 1024) * (size_t)Nx * 8));
+        size_t least = 0;   // n_fast is settled below: room for either
+        for (int fast = 0; fast < 2; ++fast) {
+            const int64_t kc = gemv_chunk(Nx, Kx, st.n_batch, fast, parts_base);
+            least = std::max(least, (size_t)st.n_batch * (size_t)((Kx + kc - 1) / kc) * (size_t)Nx * 8);
+        }
+        parts_max = std::max(parts_max, align(least));
     }
     bool any_split = false;
     for (auto &st : P->steps) any_split |= st.kernel == KK_GEMM_SPLIT || st.kernel == KK_GEMM_EMU;
@@ -1214,7 +1246,8 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             for (int d = 0; d < v.n.n; ++d) min_n = std::min(min_n, v.n.s0[d]);
             for (int d = 0; d < v.k.n; ++d) min_k = std::min(min_k, v.k.s1[d]);
             v.n_fast = min_n < min_k ? 1 : 0;
-            v.nchunks = (v.K + 1023) / 1024;
+            v.kc = gemv_chunk(v.N, v.K, st.n_batch, v.n_fast, parts_base);
+            v.nchunks = (v.K + v.kc - 1) / v.kc;
             {   // batch digits in-kernel: (vector, large operand) offsets and result offsets
                 std::vector<int> none;
                 std::vector<int64_t> sv(L, 0), sx(L, 0), sy(L, 0), zero(L, 0);
@@ -1228,6 +1261,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
                 fill_radix(&v.by, st.form.Bt, ex.data(), sy.data(), zero.data());
                 v.n_batch = (uint32_t)st.n_batch;
             }
+            v.vec4 = gemv_vec4(v);
             continue;
         }
         if (st.kernel == KK_GEMM_SPLIT || st.kernel == KK_GEMM_EMU) {
