@@ -16,13 +16,18 @@
 //     and summed indices outside the block zero;
 //   * main kernel (triples_tc_kernel), persistent, one CTA per SM: a TMA warp loads, per work
 //     item, term and chunk, the three planes of both operand tiles into a ring slot (one 2-D
-//     tensor map over all plane rows, 64-row boxes, 64-byte swizzle); one thread issues the six
+//     tensor map over all plane rows, 192-row boxes, 64-byte swizzle); one warp issues the six
 //     products (hh, hm, mh, hl, lh, mm; the dropped ml, lm, ll sum to at most 2^-23 relative) as tcgen05
 //     MMAs of 128 x 64 x 16 into one of four tensor-memory accumulators; sixteen drain warps
 //     (four per lane quadrant, 16 columns each) load the accumulator and add alpha times it into
 //     the pair-tile, the first term storing (column offsets are constants of the term's label
 //     split: one code path per split); then the energy of the pair-tile's elements inside the
 //     block, one FP64 atomic per pair-tile.
+// What bounds it: the drain (shared-memory pipe 45 %, issue slots 48 %), in step with one pair-tile's
+// terms.  Sixteen uneven blocks of extents 8 .. 32, nine terms: 12.6 ms; with the six MMAs and nine
+// 64-row boxes of a chunk issued under `lane == 0`, each of which moves its operands to uniform
+// registers first, 13.5 ms.  The barrier between two terms behind the next accumulator's load
+// (instead of in front of it) was slower, 13.2 ms: the loads then wait in the slowest warp.
 // Every wait is bounded; a wait that runs out records COMET_ERR_TIMEOUT in the status word.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -344,8 +349,8 @@ __global__ void __launch_bounds__(tc::THREADS, 1)
     };
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------- TMA producer ----------------
+        {
+            // ---------------- TMA producer (the whole warp; see elect_one) ----------------
             uint32_t rit = 0;
             bool ok = true, injected = false;
             ItemWalk walk;
@@ -358,32 +363,32 @@ __global__ void __launch_bounds__(tc::THREADS, 1)
                     const int32_t wrow = rec_row(rec, 0, item), nrow = rec_row(rec, 1, item);
                     for (int ch = 0; ch < rec.nch && ok; ++ch) {
                         const uint32_t s = rit % RING, rnd = rit / RING;
-                        if (rnd > 0 && !mbar_wait(&empty[s], (rnd - 1) & 1, tmo, abort_flag)) { ok = false; break; }
-                        mbar_arrive_expect_tx(&full[s], SLOT);
+                        if (rnd > 0 && !warp_wait(&empty[s], (rnd - 1) & 1, tmo, abort_flag)) { ok = false; break; }
+                        if (elect_one()) mbar_arrive_expect_tx(&full[s], SLOT);
                         ++rit;
                         if ((t.debug_flags & 1) && !injected && blockIdx.x == 0) {
                             injected = true;   // fault injection: this slot's loads are withheld
                             continue;
                         }
                         uint8_t *dst = ring + s * SLOT;
-#pragma unroll
-                        for (int pl = 0; pl < 3; ++pl) {
-                            const int wr = wrow + (ch * 3 + pl) * WROWS, nr = nrow + (ch * 3 + pl) * NROWS;
-                            tma_load_2d(&map, &full[s], dst + pl * WPLANE, 0, wr);
-                            tma_load_2d(&map, &full[s], dst + pl * WPLANE + BOX * ROWB, 0, wr + BOX);
-                            tma_load_2d(&map, &full[s], dst + 3 * WPLANE + pl * NPLANE, 0, nr);
+                        const int wr = wrow + ch * 3 * WROWS, nr = nrow + ch * 3 * NROWS;   // a chunk's planes adjoin
+                        if (elect_one()) {
+                            tma_load_2d(&map, &full[s], dst, 0, wr);
+                            tma_load_2d(&map, &full[s], dst + BOX * ROWB, 0, wr + BOX);
+                            tma_load_2d(&map, &full[s], dst + 3 * WPLANE, 0, nr);
                         }
+                        __syncwarp();
                     }
                 }
             }
-            if (!ok) fail();
+            if (!ok && lane == 0) fail();
             // wait (bounded) for every load still in flight before the CTA may exit
             for (uint32_t j = rit > (uint32_t)RING ? rit - RING : 0; j < rit; ++j)
                 mbar_wait(&full[j % RING], (j / RING) & 1, tmo, nullptr);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer ----------------
+        {
+            // ---------------- MMA issuer (the whole warp; see elect_one) ----------------
             constexpr uint32_t idesc = idesc_bf16_f32(WROWS, NROWS);
             uint32_t rit = 0, tcount = 0;
             bool ok = true;
@@ -396,38 +401,42 @@ __global__ void __launch_bounds__(tc::THREADS, 1)
                     const TcRec rec = load_rec(t.rec, (int64_t)item.b * a.n_terms + p);
                     const int ed = rec.ed, nch = rec.nch;
                     const uint32_t ab = tcount % NACC, rnd = tcount / NACC;
-                    if (rnd > 0 && !mbar_wait(&tempty[ab], (rnd - 1) & 1, tmo, abort_flag)) { ok = false; break; }
+                    if (rnd > 0 && !warp_wait(&tempty[ab], (rnd - 1) & 1, tmo, abort_flag)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t d = tmem_base + ab * NROWS;
                     for (int ch = 0; ch < nch; ++ch) {
                         const uint32_t s = rit % RING;
-                        if (!mbar_wait(&full[s], (rit / RING) & 1, tmo, abort_flag)) { ok = false; break; }
+                        if (!warp_wait(&full[s], (rit / RING) & 1, tmo, abort_flag)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t sa = smem_u32(ring + s * SLOT), sb = sa + 3 * WPLANE;
                         const int kn = min(KCH, ed - ch * KCH), ksteps = (kn + 15) >> 4;
-                        for (int ks = 0; ks < ksteps; ++ks) {
-                            const uint64_t ah = tile_desc(sa + ks * 32), am = tile_desc(sa + WPLANE + ks * 32),
-                                           al = tile_desc(sa + 2 * WPLANE + ks * 32);
-                            const uint64_t bh = tile_desc(sb + ks * 32), bm = tile_desc(sb + NPLANE + ks * 32),
-                                           bl = tile_desc(sb + 2 * NPLANE + ks * 32);
-                            // the small products first, hh last
-                            mma_bf16(d, am, bm, idesc, (ch > 0 || ks > 0) ? 1u : 0u);
-                            mma_bf16(d, al, bh, idesc, 1);
-                            mma_bf16(d, ah, bl, idesc, 1);
-                            mma_bf16(d, am, bh, idesc, 1);
-                            mma_bf16(d, ah, bm, idesc, 1);
-                            mma_bf16(d, ah, bh, idesc, 1);
+                        if (elect_one()) {
+                            for (int ks = 0; ks < ksteps; ++ks) {
+                                const uint64_t ah = tile_desc(sa + ks * 32), am = tile_desc(sa + WPLANE + ks * 32),
+                                               al = tile_desc(sa + 2 * WPLANE + ks * 32);
+                                const uint64_t bh = tile_desc(sb + ks * 32), bm = tile_desc(sb + NPLANE + ks * 32),
+                                               bl = tile_desc(sb + 2 * NPLANE + ks * 32);
+                                // the small products first, hh last
+                                mma_bf16(d, am, bm, idesc, (ch > 0 || ks > 0) ? 1u : 0u);
+                                mma_bf16(d, al, bh, idesc, 1);
+                                mma_bf16(d, ah, bl, idesc, 1);
+                                mma_bf16(d, am, bh, idesc, 1);
+                                mma_bf16(d, ah, bm, idesc, 1);
+                                mma_bf16(d, ah, bh, idesc, 1);
+                            }
+                            mma_commit(&empty[s]);
+                            if (ch == nch - 1) mma_commit(&tfull[ab]);   // the term's product is complete: the drain may read it
                         }
-                        mma_commit(&empty[s]);
+                        __syncwarp();
                         ++rit;
                     }
                     if (!ok) break;
-                    mma_commit(&tfull[ab]);   // the term's product is complete: the drain may read it
                 }
             }
-            if (!ok) fail();
+            if (!ok && lane == 0) fail();
             // no MMA may still write tensor memory when it is freed
-            mma_commit(mma_done);
+            if (elect_one()) mma_commit(mma_done);
+            __syncwarp();
             mbar_wait(mma_done, 0, tmo, nullptr);
         }
     } else {
@@ -558,7 +567,7 @@ cudaError_t launch_triples_tc(const Plan &P, const Args &a, TcArgs t, cudaStream
     const TriplesPlan &tp = P.tri;
     auto enc = tri_encode_fn();
     if (!enc || tp.tc_max_rows <= 0 || tp.tc_max_rows >= (int64_t(1) << 31)) return cudaErrorInvalidValue;
-    // one map over the batch region's plane rows: 32 bf16 per row, 64-row boxes, 64-byte swizzle
+    // one map over the batch region's plane rows: 32 bf16 per row, 192-row boxes, 64-byte swizzle
     CUtensorMap map;
     cuuint64_t dims[2] = {(cuuint64_t)tc::KCH, (cuuint64_t)tp.tc_max_rows};
     cuuint64_t strides[1] = {(cuuint64_t)tc::ROWB};

@@ -75,6 +75,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
     }
     return true;
 }
+// mbar_wait by a whole warp: true when every lane saw the phase end
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, uint64_t timeout_ns, volatile int *abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, timeout_ns, abort_flag));
+}
 
 // ---- CTA pairs (clusters of two) ----------------------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_rank() {

@@ -46,7 +46,7 @@ constexpr int KCH = 32;            // summed indices per plane row
 constexpr int ROWB = 64;           // bytes per plane row
 constexpr int WROWS = 128;         // rows of the operand holding label 0 (8 x 4 x 4)
 constexpr int NROWS = 64;          // rows of the other operand (4 x 4 x 4)
-constexpr int BOX = 64;            // rows per TMA box
+constexpr int BOX = 192;           // rows per TMA box: half of the wide operand's planes, all of the other's
 constexpr int WPLANE = WROWS * ROWB, NPLANE = NROWS * ROWB;
 constexpr int SLOT = 3 * (WPLANE + NPLANE);   // one (term, chunk): three planes of both operands
 constexpr int RING = 4;
