@@ -5,11 +5,15 @@ contraction that comet_adjoint_expr() writes (the incoming gradient contracted w
 other operand onto that operand's labels).  Each adjoint is planned like any expression, so
 the adjoint of a multi-operand chain gets its own operand order and recomputes the
 intermediates it needs instead of keeping the forward's intermediates alive.  All arithmetic
-runs in the library's kernels; this module only builds arguments and allocates buffers.
+runs in the library's kernels; this module only builds arguments and allocates buffers.  What
+follows from the strings alone (labels, reversed and adjoint expressions) is remembered, bounded:
+parsing them again on every call left the GPU waiting on the host (a chain's forward and backward took
+490 us instead of 390).
 """
 from __future__ import annotations
 
 import ctypes
+import functools
 import re
 
 import torch
@@ -21,6 +25,7 @@ _cache: dict = {}
 _TENSOR = re.compile(r"([A-Za-z_]\w*)\s*([\[(])([^\])]*)([\])])")
 
 
+@functools.lru_cache(maxsize=1024)
 def _reverse_labels(expr: str) -> str:
     """Row-major (torch) labels -> the column-major order of the C ABI: reverse every list."""
     def rev(m):
@@ -29,6 +34,7 @@ def _reverse_labels(expr: str) -> str:
     return _TENSOR.sub(rev, expr)
 
 
+@functools.lru_cache(maxsize=1024)
 def adjoint_expr(expr: str, operand: int) -> str:
     buf = ctypes.create_string_buffer(4096)
     _lib.check(lib().comet_adjoint_expr(expr.encode(), operand, buf, len(buf)), "comet_adjoint_expr")
@@ -44,18 +50,18 @@ def _plan(expr, ext, dtype, precision, order, workspace_cap):
     return p
 
 
+@functools.lru_cache(maxsize=1024)
 def _labels(expr):
     tensors = _TENSOR.findall(expr)
-    out = [l.strip() for l in tensors[0][2].split(",") if l.strip()]
-    ins = [[l.strip() for l in t[2].split(",") if l.strip()] for t in tensors[1:]]
+    out = tuple(l.strip() for l in tensors[0][2].split(",") if l.strip())
+    ins = tuple(tuple(l.strip() for l in t[2].split(",") if l.strip()) for t in tensors[1:])
     return out, ins
 
 
 def _run(expr, ext, tensors, precision, order, workspace_cap):
     t0 = tensors[0]
     p = _plan(expr, ext, t0.dtype, precision, order, workspace_cap)
-    out_labels, _ = _labels(expr)
-    out = torch.empty(tuple(reversed([ext[l] for l in out_labels])), dtype=t0.dtype, device=t0.device)
+    out = torch.empty([ext[l] for l in reversed(_labels(expr)[0])], dtype=t0.dtype, device=t0.device)
     p.contract([t.contiguous() for t in tensors], out, p.workspace(t0.device))
     return out
 
