@@ -23,13 +23,14 @@
 //   warp 0       TMA producer: one 3-D tensor load per operand and stage brings both planes of
 //                the CTA's 128 rows of A and bn/2 rows of B, 64 K values, 128-byte swizzled; all
 //                of a stage's loads, from both CTAs, complete on CTA 0's barrier
-//   warp 1       allocates 512 tensor-memory columns (two accumulators); in CTA 0, one lane issues
-//                tcgen05.mma.cta_group::2 (M=256, N=bn, K=16) and commits to both CTAs
+//   warp 1       allocates 512 tensor-memory columns (two to four accumulators, see NBUF); in CTA 0
+//                the whole warp runs the loop and one elected lane issues tcgen05.mma.cta_group::2
+//                (M=256, N=bn, K=16) and commits to both CTAs
 //   warps 4..15  epilogue: each owns one tensor-memory lane quadrant and one third of the
 //                columns; drains an accumulator after every chunk into register sums (64 columns
 //                in two levels: 128 registers of a thread's 160) while the MMAs fill the other one,
 //                and at the end of the tile stores through the output's strides (the output
-//                permutation of TTGT folded in)
+//                permutation of TTGT folded in; through shared memory where its runs lie along N)
 //   3-stage shared-memory ring (56 KB per stage and CTA at bn = 192).
 // What bounds it: the power cap at large sizes.  M = N = K = 12288: 7.0 ms = 1.6 PFLOP/s of MMA
 // (six bf16 products: 10.7-10.9 ms); at middle sizes the hand-over of an accumulator per chunk (see NBUF).
