@@ -36,8 +36,8 @@
 // (six bf16 products: 10.7-10.9 ms); at middle sizes the hand-over of an accumulator per chunk (see NBUF).
 // Why pairs: with one CTA per 128 x 256 tile a stage reads 144 KB of operands from shared memory
 // and fills 96 KB per 1536 MMA cycles, 160 bytes per clock against the SM's 128; in a pair each
-// CTA holds half of B (bn = 192: 84 + 56 KB per 1152 cycles, 121).  Tiles of 240 and 256 columns run
-// 5 % faster at 12288^3 (7.0 ms) but leave no registers for the second level of sums.
+// CTA holds half of B (bn = 192: 84 + 56 KB per 1152 cycles, 121).  Tiles of 240 and 256 columns ran
+// 5 % faster at 12288^3 (before the warp-wide issue) but leave no registers for the second level of sums.
 // Every wait is bounded (%globaltimer); on expiry the CTA records COMET_ERR_TIMEOUT in the
 // status word, drains its own copies in flight, frees its tensor memory and returns.
 #include <cuda.h>
