@@ -367,7 +367,7 @@ static comet_status_t run_host_pipe(const Plan &P, int n_calls, const void *cons
         }
     } r;
     const int n = h.n_chunks, nw = h.w_n;
-    if (n + nw > 32) return COMET_ERR_INTERNAL;   // one scale word per slice in the 256-byte region
+    if (n + nw > 31) return COMET_ERR_INTERNAL;   // one scale word per slice in the 256-byte region, and a slot
     cudaError_t e = cudaStreamCreateWithFlags(&r.cin, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&r.cout, cudaStreamNonBlocking);
     // per call: start, end, X copies, column results, W copies, blocks; across calls: the
@@ -479,8 +479,8 @@ static comet_status_t run_host_pipe(const Plan &P, int n_calls, const void *cons
             part.x = src;
             part.n = n_elems;
             part.view = 0;
-            part.blocks = absmax_blocks(n_elems, (int)es, st.n_slots);
-            part.slots = w + st.ws_slots;
+            part.blocks = absmax_blocks(n_elems, (int)es, h.n_slots);
+            part.slots = w + h.ws_slots;
             ee = launch_absmax(part, none, (int)es, s);
         }
         if (ee == cudaSuccess) {

@@ -705,6 +705,15 @@ void setup_host_pipe(Plan *P, int64_t es, int want, int want_w) {
         prepass_params(st, sw.labels, label_strides(sw.labels, ew), 0, wrows, ew, es, &h.w_pre[i], &h.w_pre_vec[i],
                        &h.w_pre_vout[i]);
     }
+    // A slice's abs-max slots: the step's, unless those lie beside the scale words (the planner's fallback);
+    // the pipe keeps a scale word for every slice there, and its slots are what these leave of the 32.
+    h.ws_slots = st.ws_slots;
+    h.n_slots = st.n_slots;
+    if (st.ws_slots < st.ws_scales + 256) {
+        const uint32_t words = (uint32_t)(h.n_chunks + h.w_n);   // at most 31, see the candidates
+        h.ws_slots = st.ws_scales + 8 * words;
+        h.n_slots = 32 - words;
+    }
     h.ok = true;
     P->pipe = h;
 }
@@ -1182,8 +1191,8 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
     for (auto &st : P->steps) any_split |= st.kernel == KK_GEMM_SPLIT || st.kernel == KK_GEMM_EMU;
     // after the parts: 256 bytes of scale words (slices of the host pipeline have one each) and the
     // slots of the abs-max pass, one per block and operand; where those would put the plan past
-    // the library's static scratch, the 14 per operand that the scale words leave room for (a
-    // host-pipelined plan is larger than that scratch or its slices few)
+    // the library's static scratch, the 14 per operand that the step's two scale words leave room
+    // for (the host pipeline, with more scale words and one operand at a time, places its own)
     const size_t scales_end = parts_base + parts_max + 256;
     const bool room = scales_end > COMET_NOALLOC_MAX_BYTES || scales_end + 16 * kSlots <= COMET_NOALLOC_MAX_BYTES;
     for (auto &st : P->steps) {

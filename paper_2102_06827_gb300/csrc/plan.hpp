@@ -131,6 +131,8 @@ struct HostPipe {
     std::vector<int> blocks;     // GEMM order: i * n_chunks + j
     bool blockwise = false;      // results go back block by block
     double model_s[2] = {0, 0};  // modelled seconds: unpipelined, pipelined
+    size_t ws_slots = 0;         // abs-max slots of the slice in work (8-byte words beside no scale word)
+    uint32_t n_slots = 0;
 };
 
 // Fused triples accumulation (comet_plan_triples): T_b = sum_p alpha_p X_bp * Y_bp over terms
