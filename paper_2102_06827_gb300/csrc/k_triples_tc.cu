@@ -206,6 +206,13 @@ __device__ __forceinline__ void add_exact(float &hi, float &lo, float h, float l
     hi = s;
 }
 
+// the warp's sum, in FP64
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 // one drain warp's 16 columns of a term's product for this thread's row: column n = 16 colq +
 // c0 + 4 c1 sits at the narrow labels' coordinates (c0, c1, colq); the first term stores, the
 // others add (all loads before the stores: the 16 slots are distinct)
@@ -315,6 +322,7 @@ __global__ void __launch_bounds__(tc::THREADS, 1)
     int *s_geo = reinterpret_cast<int *>(s_red + DRAIN_WARPS);     // per term: pair-tile strides of
                                                                    // the wide labels 1, 2; narrow mask
     __shared__ float Tsh[TSZ];                                      // the pair-tile
+    __shared__ double s_wide[DRAIN_WARPS];                          // partial sums beyond FP32's range
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t tmo = (uint64_t)t.timeout_ns;
@@ -524,10 +532,13 @@ __global__ void __launch_bounds__(tc::THREADS, 1)
                     hi += in ? v : 0.0f;
                 }
             }
-            // the 512 threads' sums with their exact rounding errors beside them: as accurate as FP64
-            // (2^-48), whose additions the SM does at two a clock (2560 of them a pair-tile took 4 % of it)
+            // the 512 threads' sums with their exact rounding errors beside them (relative error 2^-47), not in
+            // FP64, whose additions the SM does at two a clock (2560 of them a pair-tile took 4 % of it).
+            // Where that leaves FP32's range (an error term is then not a number) the sums are added in FP64.
+            const float part = hi;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) add_exact(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
+            if (!(fabsf(hi) < INFINITY)) s_wide[warp - 2] = warp_sum(part);   // in all lanes or in none: hi is the same in each
             if (lane == 0) s_red[warp - 2] = make_float2(hi, lo);
             named_bar_sync(1, 32 * DRAIN_WARPS);   // the pair-tile is read; partial sums are in
             if (warp == 2) {
@@ -536,7 +547,12 @@ __global__ void __launch_bounds__(tc::THREADS, 1)
                 lo = v.y;
 #pragma unroll
                 for (int o = DRAIN_WARPS / 2; o > 0; o >>= 1) add_exact(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
-                if (lane == 0 && hi != 0.0f) atomicAdd(a.energies + item.b, (double)hi + (double)lo);
+                if (!(fabsf(hi) < INFINITY)) {
+                    const double sum = warp_sum(lane >= DRAIN_WARPS ? 0.0 : fabsf(v.x) < INFINITY ? (double)v.x + (double)v.y : s_wide[lane]);
+                    if (lane == 0) atomicAdd(a.energies + item.b, sum);
+                } else if (lane == 0 && (hi != 0.0f || lo != 0.0f)) {
+                    atomicAdd(a.energies + item.b, (double)hi + (double)lo);
+                }
             }
         }
     }
