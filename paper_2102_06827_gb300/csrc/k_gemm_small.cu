@@ -27,6 +27,7 @@
 #include "launch.h"
 #include "params.h"
 #include "split.cuh"
+#include "split_schedule.h"
 
 namespace comet {
 
@@ -250,7 +251,7 @@ cudaError_t launch_gemm_small(const GemmParams &p, bool a_kcontig, bool b_kconti
     using namespace sg;
     if (p.M == 0 || p.N == 0) return cudaSuccess;
     const dim3 grid((p.M + TM - 1) / TM, (p.N + TM - 1) / TM);
-    if (grid.y > 65535) return cudaErrorInvalidConfiguration;
+    if (!small_gemm_fits(p.N)) return cudaErrorInvalidConfiguration;   // the planner does not send such a step here
     if (a_kcontig && b_kcontig) launch_pdl(gemm_small_kernel<true, true>, grid, T, SMEM, s, p);
     else if (a_kcontig) launch_pdl(gemm_small_kernel<true, false>, grid, T, SMEM, s, p);
     else if (b_kcontig) launch_pdl(gemm_small_kernel<false, true>, grid, T, SMEM, s, p);

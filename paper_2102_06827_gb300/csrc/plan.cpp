@@ -1126,7 +1126,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
                 return std::max(contiguous_run(rows, t, P->extent), contiguous_run(st.form.K, t, P->extent));
             };
             const bool long_runs = run(sm, st.form.M) >= 16 && run(sn, st.form.N) >= 16;
-            st.small = P->dtype == COMET_F32 && opts.ksplit <= 0 && !(opts.debug_flags & 1) &&
+            st.small = P->dtype == COMET_F32 && opts.ksplit <= 0 && !(opts.debug_flags & 1) && small_gemm_fits((uint64_t)rows_b) &&
                        small_gemm_us((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, long_runs) < sch.us + 8.0;
             bk = (size_t)split_partial_bytes((uint64_t)rows_a, (uint64_t)rows_b, sch);
             const int64_t tiles = ((rows_a + 127) / 128) * ((rows_b + 255) / 256), tail = tiles % 152;

@@ -92,6 +92,9 @@ inline double small_gemm_us(uint64_t M, uint64_t N, uint64_t K, bool long_runs) 
     return 3.0 + (double)((tiles + 151) / 152) * (900.0 + (double)K * (long_runs ? 22.0 : 42.0)) / 1900.0;
 }
 
+// Whether its grid takes the size: N runs along y (the planner's own forms put the longer side on M)
+inline bool small_gemm_fits(uint64_t N) { return (N + 15) / 16 <= 65535; }
+
 // The emulated-FP64 GEMM: whole-K tiles of 128 x 80 in full waves over the SMs, the tiles left over in
 // K slices of whole chunks (192 values) whose int64 partial sums a second kernel adds.
 constexpr int kEmuBM = 128, kEmuBN = 80, kEmuChunk = 192;

@@ -73,3 +73,13 @@ def test_infinite_element_beside_tiny_ones():
     C, _ = run(A, B, 1e30)
     ref = 1e30 * (f32(A).T @ f32(B))
     assert np.all(np.isinf(C[2])) and np.allclose(C[[0, 1, 3]], ref[[0, 1, 3]], rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("m,n,k", [(8, 1048560, 8), (8, 1048561, 8), (2, 1100000, 3)])
+def test_long_dimension_in_either_form(m, n, k, form):
+    # the one-launch kernel takes N up to 65535 tiles of 16; the forms put either dimension there
+    rng = np.random.default_rng(n + form)
+    A, B = f32(rng.normal(size=(k, m))), f32(rng.normal(size=(k, n)))
+    C, step = run(A, B, form=form)
+    assert normwise(C, A.T @ B) <= 6e-7
