@@ -103,7 +103,7 @@ typedef struct {
     int form;                   /* -1 = planner's choice; k >= 0 = k-th enumerated TTGT form
                                    of every binary step (for the permutation ablation) */
     int64_t kc;                 /* split path: an upper limit of the K elements per accumulation
-                                   chunk; the kernel's chunks are 32 or 64 whatever its value */
+                                   chunk (0 = none).  Chunks are 32 or 64: a limit below 64 gives 32 */
     int64_t timeout_ms;         /* device-side wait limit; 0 = default (2000 ms) */
     int debug_flags;            /* bit 0: withhold one operand load in the split GEMM so that
                                    its wait runs out (fault-injection test); bit 3, builds with

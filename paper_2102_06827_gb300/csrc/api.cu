@@ -302,7 +302,7 @@ static comet_status_t run_plan(const Plan &P, const void *const *inputs, void *o
             } else {
                 ProfScope ps(PK_SPLIT, stream);
                 e = launch_gemm_split(g, w + st.ws_parts_a, w + st.ws_parts_b, st.kpad, sc_a, sc_b,
-                                      es, P.opts.debug_flags, stream, st.want_ksplit,
+                                      P.opts.kc, es, P.opts.debug_flags, stream, st.want_ksplit,
                                       reinterpret_cast<float *>(w + st.ws_ksplit), (int64_t)st.ksplit_bytes);
                 if (e != cudaSuccess) return cuda_status(e, "split gemm kernel");
             }
@@ -560,7 +560,7 @@ static comet_status_t run_host_pipe(const Plan &P, int n_calls, const void *cons
                                     reinterpret_cast<long long *>(w + st.ws_ksplit), (int64_t)st.ksplit_bytes);
             } else {
                 ProfScope ps(PK_SPLIT, s);
-                e = launch_gemm_split(g, pa, pb, st.kpad, sa, sb, (int)es, P.opts.debug_flags, s,
+                e = launch_gemm_split(g, pa, pb, st.kpad, sa, sb, P.opts.kc, (int)es, P.opts.debug_flags, s,
                                       st.want_ksplit, reinterpret_cast<float *>(w + st.ws_ksplit),
                                       (int64_t)st.ksplit_bytes);
             }

@@ -585,12 +585,12 @@ static void launch_split_kernel(const CUtensorMap &ta, const CUtensorMap &tb, co
 
 cudaError_t launch_gemm_split(const GemmParams &p, const void *parts_a, const void *parts_b,
                               int64_t kpad, const void *scale_a, const void *scale_b,
-                              int out_bytes, int debug_flags, cudaStream_t s,
+                              int64_t kc, int out_bytes, int debug_flags, cudaStream_t s,
                               uint32_t want_ksplit, float *partial, int64_t partial_bytes) {
     using namespace split;
     if (p.M == 0 || p.N == 0) return cudaSuccess;
     const uint32_t pairs = (uint32_t)std::max(1, sm_count() / 2);
-    const SplitSchedule sch = split_schedule(p.M, p.N, p.K, pairs, want_ksplit, partial ? partial_bytes : 0);
+    const SplitSchedule sch = split_schedule(p.M, p.N, p.K, pairs, want_ksplit, partial ? partial_bytes : 0, kc);
     CUtensorMap ta, tb;
     if (!make_map(&ta, parts_a, p.M, p.K, (uint64_t)kpad, BM)) return cudaErrorInvalidValue;
     if (!make_map(&tb, parts_b, p.N, p.K, (uint64_t)kpad, sch.bn / 2)) return cudaErrorInvalidValue;
@@ -604,7 +604,7 @@ cudaError_t launch_gemm_split(const GemmParams &p, const void *parts_a, const vo
     x.ksplit = sch.ksplit;
     x.kslice_chunks = (x.nch + sch.ksplit - 1) / sch.ksplit;
     x.items = x.m_tiles * x.n_tiles * x.ksplit;
-    split_chunks(x.kslice_chunks, &x.chunk_steps, &x.group);
+    split_chunks(x.kslice_chunks, kc, &x.chunk_steps, &x.group);
     x.partial = partial;
     x.dbg_p = dbg_range(partial, split_partial_bytes(p.M, p.N, sch));
     // along columns where the N group's first label is C's stride-1 label (and the M group's is not)

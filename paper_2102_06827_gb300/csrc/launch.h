@@ -67,11 +67,11 @@ cudaError_t launch_gemm_small(const GemmParams &p, bool a_kcontig, bool b_kconti
 cudaError_t launch_fill(void *out, int64_t n, double value, int elem_bytes, cudaStream_t s);
 
 // Two FP16 planes per operand.  want_ksplit: 0 = K slices and tile width by split_schedule, k = k
-// slices; FP32 partials of the slices in `partial` (as many as fit partial_bytes), summed by a
+// slices; kc: upper limit of a chunk's K values (0 = none); FP32 partials of the slices in `partial` (as many as fit partial_bytes), summed by a
 // reduce kernel into C.
 cudaError_t launch_gemm_split(const GemmParams &p, const void *parts_a, const void *parts_b,
                               int64_t kpad, const void *scale_a, const void *scale_b,
-                              int out_bytes, int debug_flags, cudaStream_t s,
+                              int64_t kc, int out_bytes, int debug_flags, cudaStream_t s,
                               uint32_t want_ksplit, float *partial, int64_t partial_bytes);
 
 // `partial`: room for the int64 sums of K slices (emu_schedule; as many as fit partial_bytes)

@@ -560,7 +560,7 @@ void setup_host_pipe(Plan *P, int64_t es, int want, int want_w) {
     auto t_block = [&](int64_t lx, int64_t lw) {   // one GEMM block of lx x lw label indices
         const int64_t r = h.rows_inner * lx, rw = h.w_rows_inner * lw, M = h.side ? rw : r, N = h.side ? r : rw;
         return emu ? (double)((((M + tm - 1) / tm) * ((N + tn - 1) / tn) + 151) / 152) * t_tile
-                   : 1e-6 * split_schedule((uint64_t)M, (uint64_t)N, (uint64_t)st.kpad, 76, 1, 0).us;
+                   : 1e-6 * split_schedule((uint64_t)M, (uint64_t)N, (uint64_t)st.kpad, 76, 1, 0, P->opts.kc).us;
     };
     const int64_t xu = h.x_inner * h.x_outer, wu = h.w_inner * h.w_outer;
     // slice boundaries: n slices, the first one 1/ramp of an equal slice, the rest equal (the
@@ -1038,7 +1038,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             const std::vector<int> &lm = swap ? sb.labels : sa.labels, &ln = swap ? sa.labels : sb.labels;
             const double t_split = kernel != KK_GEMM_SPLIT ? 0.0 : 1e-6 * split_schedule(
                 (uint64_t)prod_ext(P->extent, gm), (uint64_t)prod_ext(P->extent, gn), (uint64_t)prod_ext(P->extent, K),
-                76, 0, 64 << 20).us;
+                76, 0, 64 << 20, opts.kc).us;
             auto om = group_orders(gm, {&sc.labels, &lm});
             auto on = group_orders(gn, {&sc.labels, &ln});
             auto ok = group_orders(K, {&lm, &ln});
@@ -1114,9 +1114,13 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             least = align((size_t)6 * rows_a * st.kpad) + align((size_t)6 * rows_b * st.kpad);
             st.want_ksplit = opts.ksplit > 0 ? (uint32_t)opts.ksplit : 0;
             const SplitSchedule sch = split_schedule((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, 76,
-                                                     st.want_ksplit, room_for(least));
+                                                     st.want_ksplit, room_for(least), opts.kc);
             st.ksplit = sch.ksplit;
             st.tile_n = sch.bn;
+            const uint32_t stages = (uint32_t)((Kx + kSplitBK - 1) / kSplitBK);
+            uint32_t steps, group;
+            split_chunks((stages + sch.ksplit - 1) / sch.ksplit, opts.kc, &steps, &group);
+            st.chunk = 16 * steps;
             // one launch on the FP32 pipes where that is modelled faster than the split form's chain
             // (about 8 us of pre-passes and launches around its GEMM); asking for K slices or for the
             // fault injection keeps the split form
@@ -1348,7 +1352,7 @@ std::string describe_plan(const Plan &P) {
               << ",\"n_forms\":" << s.n_forms << ",\"form_index\":" << s.form_index
               << ",\"cost_s\":" << s.form.cost << ",\"pre_bytes\":" << s.form.pre_bytes
               << ",\"eff_store\":" << s.form.eff_store << ",\"flops\":" << s.flops
-              << ",\"ksplit\":" << s.ksplit << ",\"tile_n\":" << s.tile_n << ",\"small\":" << (s.small ? "true" : "false");
+              << ",\"ksplit\":" << s.ksplit << ",\"tile_n\":" << s.tile_n << ",\"chunk\":" << s.chunk << ",\"small\":" << (s.small ? "true" : "false");
             if (s.kernel == KK_GEMM_SPLIT)
                 o << ",\"tail_tiles\":" << s.tail_tiles << ",\"tail_slices\":" << s.tail_slices;
         }

@@ -78,6 +78,7 @@ struct Step {
     bool small = false;          // split GEMM of FP32 operands: runs as one launch (k_gemm_small.cu)
     uint32_t ksplit = 1, tile_n = 0;   // split GEMM: K slices and tile width on 152 SMs (the launch
                                        // makes the same choice from the device's own count)
+    uint32_t chunk = 0;          // split GEMM: K values per accumulation chunk
     size_t ws_ksplit = 0;        // workspace offset of the slices' FP32 partials
     size_t ksplit_bytes = 0;     // their size
     uint32_t tail_tiles = 0, tail_slices = 1;   // description: what 128 x 256 tiles leave over after

@@ -19,11 +19,12 @@ struct SplitSchedule {
 
 // Accumulation of a K slice of `stages` stages: K steps of 16 values per chunk in tensor memory (which
 // truncates: short chunks lose less, but each costs a drain) and chunks per first-level sum of
-// the epilogue (about the square root of the chunks, so that neither level adds many terms).
-inline void split_chunks(uint32_t stages, uint32_t *steps, uint32_t *group) {
+// the epilogue (about the square root of the chunks, so that neither level adds many terms).  kc: the
+// caller's upper limit of a chunk's K values (0 = none); 32 is the least there is.
+inline void split_chunks(uint32_t stages, int64_t kc, uint32_t *steps, uint32_t *group) {
     // 32 values up to K = 4096 (12 % more of the GEMM's time at 1633^3, error 1.43 -> 1.23e-7), 64 beyond
     // (8.6 against 7.7 ms at 12288^3, where the sums' own rounding is as large)
-    *steps = stages <= 64 ? 2 : 4;
+    *steps = stages <= 64 || (kc > 0 && kc < 64) ? 2 : 4;
     const uint32_t n = stages * (4 / *steps);
     uint32_t g = 1;
     while (g * g < n) ++g;
@@ -44,14 +45,14 @@ inline uint32_t split_chunks_of(uint32_t stages, uint32_t steps, uint64_t K) {
 }
 
 // The schedule with the least modelled time over the tile widths and K slices whose partial
-// sums fit `partial_limit` bytes.  want_ksplit: 0 = free, k = as near to k slices as K allows.
+// sums fit `partial_limit` bytes.  want_ksplit: 0 = free, k = as near to k slices as K allows; kc as above.
 // The model, in clocks at 1.9 GHz, from kernel times on 1633^3, 2700^3, 4864 x 960 x 4800, 200000 x 48 x
 // (96, 160) and 200000 x 192 x 48 at every width: a stage of 64 K values takes 1300 / 1420 / 1860 / 2150
 // (widths 48 / 96 / 144 / 192) in chunks of 32 and 1000 / 1130 / 1320 / 1480 in chunks of 64, a tile 2000 +
 // 26 a column around its stages, or 4700 in all for a narrow tile of at most three chunks; 3000 once; K
 // slices add a launch and their partial sums' traffic.
 inline SplitSchedule split_schedule(uint64_t M, uint64_t N, uint64_t K, uint32_t pairs, uint32_t want_ksplit,
-                                    int64_t partial_limit) {
+                                    int64_t partial_limit, int64_t kc = 0) {
     static const double stage32[4] = {1300, 1420, 1860, 2150}, stage64[4] = {1000, 1130, 1320, 1480};
     const uint64_t mt = (M + kSplitBM - 1) / kSplitBM;
     const uint32_t nch = (uint32_t)std::max<uint64_t>(1, (K + kSplitBK - 1) / kSplitBK);
@@ -69,7 +70,7 @@ inline SplitSchedule split_schedule(uint64_t M, uint64_t N, uint64_t K, uint32_t
             const int64_t pb = split_partial_bytes(M, N, s);
             if (pb > partial_limit) continue;
             uint32_t steps, group;
-            split_chunks(per, &steps, &group);
+            split_chunks(per, kc, &steps, &group);
             const double waves = (double)((tiles * s.ksplit + pairs - 1) / pairs);
             const bool narrow = w == 0 && s.ksplit == 1 && split_chunks_of(nch, steps, K) <= 3;
             const double tile = narrow ? 4700.0 : per * (steps == 2 ? stage32 : stage64)[w] + 2000.0 + 26.0 * bn;
@@ -79,7 +80,7 @@ inline SplitSchedule split_schedule(uint64_t M, uint64_t N, uint64_t K, uint32_t
         }
     }
     // more slices asked for than their partial sums may take: the most that fit
-    if (!have && want_ksplit > 1) return split_schedule(M, N, K, pairs, want_ksplit - 1, partial_limit);
+    if (!have && want_ksplit > 1) return split_schedule(M, N, K, pairs, want_ksplit - 1, partial_limit, kc);
     return best;
 }
 

@@ -25,3 +25,10 @@ def test_one_launch_kernel_only_where_its_grid_takes_the_size(m, n, k, form):
     st = step(m, n, k, form=form)
     long_n = (n if st["N"] == ["n"] else m) > 16 * 65535
     assert not (st["small"] and long_n)
+
+
+@pytest.mark.parametrize("kc,chunk", [(0, 64), (1, 32), (32, 32), (63, 32), (64, 64), (1024, 64)])
+def test_chunk_limit(kc, chunk):
+    # long sums take chunks of 64 unless the caller asks for shorter ones
+    assert step(512, 512, 6000, kc=kc, ksplit=1)["chunk"] == chunk
+    assert step(512, 512, 4096, kc=kc, ksplit=1)["chunk"] == 32
