@@ -1116,6 +1116,7 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             const SplitSchedule sch = split_schedule((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, 76,
                                                      st.want_ksplit, room_for(least), opts.kc);
             st.ksplit = sch.ksplit;
+            if (st.want_ksplit) st.want_ksplit = sch.ksplit;   // what fits, so that no launch looks for it again
             st.tile_n = sch.bn;
             const uint32_t stages = (uint32_t)((Kx + kSplitBK - 1) / kSplitBK);
             uint32_t steps, group;

@@ -74,7 +74,7 @@ struct Step {
     size_t ws_slots = 0;         // abs-max slots of A, then of B: n_slots 8-byte words each
     uint32_t n_slots = 0;
     int64_t kpad = 0;
-    uint32_t want_ksplit = 0;    // split GEMM: the caller's K slices (0 = free)
+    uint32_t want_ksplit = 0;    // split GEMM: the caller's K slices, as many as there can be (0 = free)
     bool small = false;          // split GEMM of FP32 operands: runs as one launch (k_gemm_small.cu)
     uint32_t ksplit = 1, tile_n = 0;   // split GEMM: K slices and tile width on 152 SMs (the launch
                                        // makes the same choice from the device's own count)

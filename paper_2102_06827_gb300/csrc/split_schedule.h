@@ -58,29 +58,29 @@ inline SplitSchedule split_schedule(uint64_t M, uint64_t N, uint64_t K, uint32_t
     const uint32_t nch = (uint32_t)std::max<uint64_t>(1, (K + kSplitBK - 1) / kSplitBK);
     SplitSchedule best;
     bool have = false;
-    for (uint32_t w = 0; w < 4; ++w) {
-        const uint32_t bn = 48 * (w + 1);
-        const uint64_t tiles = mt * ((N + bn - 1) / bn);
-        const uint32_t k_lo = want_ksplit ? std::min(want_ksplit, nch) : 1, k_hi = want_ksplit ? k_lo : std::min(16u, nch);
-        for (uint32_t k = k_lo; k <= k_hi; ++k) {
-            SplitSchedule s;
-            const uint32_t per = (nch + k - 1) / k;
-            s.bn = bn;
-            s.ksplit = (nch + per - 1) / per;   // every slice holds at least one stage
-            const int64_t pb = split_partial_bytes(M, N, s);
-            if (pb > partial_limit) continue;
-            uint32_t steps, group;
-            split_chunks(per, kc, &steps, &group);
-            const double waves = (double)((tiles * s.ksplit + pairs - 1) / pairs);
-            const bool narrow = w == 0 && s.ksplit == 1 && split_chunks_of(nch, steps, K) <= 3;
-            const double tile = narrow ? 4700.0 : per * (steps == 2 ? stage32 : stage64)[w] + 2000.0 + 26.0 * bn;
-            s.us = (3000.0 + waves * tile) / 1900.0;
-            if (s.ksplit > 1) s.us += 3.0 + (double)pb / 2.0e6;   // written and read back, mostly in L2
-            if (!have || s.us < best.us * (1 - 1e-9)) { best = s; have = true; }
+    uint32_t k_lo = want_ksplit ? std::min(want_ksplit, nch) : 1, k_hi = want_ksplit ? k_lo : std::min(16u, nch);
+    for (; !have && k_lo > 0; k_hi = --k_lo) {   // once, or down to as many slices as their partial sums may take
+        for (uint32_t w = 0; w < 4; ++w) {
+            const uint32_t bn = 48 * (w + 1);
+            const uint64_t tiles = mt * ((N + bn - 1) / bn);
+            for (uint32_t k = k_lo; k <= k_hi; ++k) {
+                SplitSchedule s;
+                const uint32_t per = (nch + k - 1) / k;
+                s.bn = bn;
+                s.ksplit = (nch + per - 1) / per;   // every slice holds at least one stage
+                const int64_t pb = split_partial_bytes(M, N, s);
+                if (pb > partial_limit) continue;
+                uint32_t steps, group;
+                split_chunks(per, kc, &steps, &group);
+                const double waves = (double)((tiles * s.ksplit + pairs - 1) / pairs);
+                const bool narrow = w == 0 && s.ksplit == 1 && split_chunks_of(nch, steps, K) <= 3;
+                const double tile = narrow ? 4700.0 : per * (steps == 2 ? stage32 : stage64)[w] + 2000.0 + 26.0 * bn;
+                s.us = (3000.0 + waves * tile) / 1900.0;
+                if (s.ksplit > 1) s.us += 3.0 + (double)pb / 2.0e6;   // written and read back, mostly in L2
+                if (!have || s.us < best.us * (1 - 1e-9)) { best = s; have = true; }
+            }
         }
     }
-    // more slices asked for than their partial sums may take: the most that fit
-    if (!have && want_ksplit > 1) return split_schedule(M, N, K, pairs, want_ksplit - 1, partial_limit, kc);
     return best;
 }
 

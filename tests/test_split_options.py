@@ -32,3 +32,13 @@ def test_chunk_limit(kc, chunk):
     # long sums take chunks of 64 unless the caller asks for shorter ones
     assert step(512, 512, 6000, kc=kc, ksplit=1)["chunk"] == chunk
     assert step(512, 512, 4096, kc=kc, ksplit=1)["chunk"] == 32
+
+
+@pytest.mark.parametrize("ksplit", [1000, 2 ** 31 - 1])
+def test_any_number_of_k_slices_is_planned_at_once(ksplit):
+    # more slices than K has stages, and partial sums that do not fit: the most that fit, without counting down
+    t = time.perf_counter()
+    st = step(1 << 14, 1 << 14, 4096, ksplit=ksplit)
+    assert time.perf_counter() - t < 5.0
+    assert 1 <= st["ksplit"] <= 64
+    assert st["ksplit"] == step(1 << 14, 1 << 14, 4096, ksplit=64)["ksplit"]
