@@ -85,8 +85,8 @@ struct SplitArgs {
     uint32_t chunk_steps;        // K steps of 16 per accumulation chunk (4 or 2)
     uint32_t group;              // chunks per first-level sum
     int n_fast;                  // C's stride-1 label is in the N group: a warp's stores run along columns
-    float *partial;              // per slice, tile and CTA bn x 128 partial sums (scaled by
-                                 // 2^(eA+eB)), [slice][tile][CTA][column][row], row fastest
+    float *partial;              // per slice, tile and CTA bn x 128 partial sums (of the scaled
+                                 // operands), [slice][tile][CTA][column][row], row fastest
     DbgRange dbg_p;              // debug builds: the partial sums' buffer
     int debug_flags;
     const void *scale_a;         // bits of max |A|, max |B| (input precision)
@@ -405,14 +405,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
             const uint32_t ml = quad * 32 + lane, m = mt * (2 * BM) + rank * BM + ml;
             const uint32_t n0 = nt * x.bn + g0;
             const int n_here = (int)min(gn, p.N > n0 ? p.N - n0 : 0u);
-            if constexpr (KSPLIT) {   // K slice partial: scaled sums to the tile's slot, row fastest (coalesced)
+            if constexpr (KSPLIT) {   // K slice partial: the sums to the tile's slot, row fastest (coalesced)
                 if (m < p.M) {
-                    const float sp = (float)ldexp(1.0, e_sum);
                     float *P = x.partial + ((((size_t)ks * tiles + t % tiles) * 2 + rank) * x.bn + g0) * BM + ml;
 #pragma unroll
                     for (int j = 0; j < GN; ++j)
                         if (j < n_here && dbg_ok(x.dbg_p, P + (size_t)j * BM, 4, p.status))
-                            P[(size_t)j * BM] = sp * result(j);
+                            P[(size_t)j * BM] = result(j);
                 }
             } else if (x.n_fast) {
                 // through shared memory, 16 columns at a time, so that sixteen lanes store one row's
@@ -478,15 +477,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
     if (warp == 1) tmem_dealloc_pair(tmem_base, TMEM_COLS);
 }
 
-// K-slice partials -> C: C[m, n] = alpha * sum_ks P[ks][tile][CTA][n][m] (+ beta C), through C's
-// strides.  A block takes 32 columns of one CTA's 128 rows: a thread keeps one row (its offset
-// is worked out once) and walks 16 columns, whose offsets the block tabulates, so reads and stores
+// K-slice partials -> C: C[m, n] = alpha 2^(eA+eB) sum_ks P[ks][tile][CTA][n][m] (+ beta C), through
+// C's strides.  The operands' scale comes in here, with alpha, and not into the FP32 partials, whose range it
+// may leave (FP64 operands, or an alpha that brings the result back).
+// A block takes 24 columns of one CTA's 128 rows: a thread keeps one row (its offset
+// is worked out once) and walks 12 columns, whose offsets the block tabulates, so reads and stores
 // run along the rows.  The slices are added with an exact error term (two-sum) in FP32: FP64 adds
 // run at 1/64 of that rate here (39 us of 163 on a 1633^3 contraction with two slices).
 template <typename TOut>
 __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmParams p, const SplitArgs x) {
     using namespace split;
     __shared__ int64_t c_col[STRIP];
+    __shared__ int s_exp;
     const uint32_t strips = x.bn / STRIP;
     const uint32_t strip = blockIdx.x % strips, cta = blockIdx.x / strips, tile = cta >> 1, rank = cta & 1;
     uint32_t mt, nt;
@@ -500,8 +502,15 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmParams p, c
     int64_t r0 = 0, c_row = 0;
     if (m < p.M) radix_offsets(p.ma, m, r0, c_row);
     pdl_wait();
+    if (threadIdx.x == 0)
+        s_exp = half_exponent<TOut>(scale_exponent<TOut>(x.scale_a)) + half_exponent<TOut>(scale_exponent<TOut>(x.scale_b));
     __syncthreads();
     if (m >= p.M) return;
+    const int e_sum = s_exp;
+    // plain FP32 results: one product with a normal power of two; everything else in FP64
+    const bool plain = sizeof(TOut) == 4 && p.alpha == 1.0 && p.beta == 0.0 && e_sum >= -126 && e_sum <= 127;
+    const float sc = plain ? __int_as_float((e_sum + 127) << 23) : 0.0f;
+    const double scale = plain ? 0.0 : ldexp(p.alpha, e_sum);
     const size_t slice = (size_t)x.m_tiles * x.n_tiles * 2 * x.bn * BM;
     const float *P = x.partial + ((size_t)cta * x.bn + strip * STRIP) * BM + ml;
 #pragma unroll 4
@@ -518,10 +527,10 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmParams p, c
         TOut *c = reinterpret_cast<TOut *>(p.C) + c_row + c_col[j];
         if (!dbg_ok(p.dbg_c, c, (int)sizeof(TOut), p.status)) continue;
         if (!(fabsf(s) < INFINITY)) lo = 0.0f;   // the error term of an infinite sum is not a number
-        if (sizeof(TOut) == 4 && p.alpha == 1.0 && p.beta == 0.0) {
-            *c = (TOut)(s + lo);
+        if (plain) {
+            *c = (TOut)(sc * (s + lo));
         } else {
-            const double r = p.alpha * ((double)s + (double)lo);
+            const double r = scale * ((double)s + (double)lo);
             *c = (TOut)(p.beta != 0.0 ? r + p.beta * (double)*c : r);
         }
     }
