@@ -165,6 +165,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
              *mma_done = tempty + MAXBUF;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    volatile uint32_t *issued = tmem_slot + 2;   // stages that CTA 0 and CTA 1 of the pair have loaded
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
@@ -253,7 +254,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
                     tma_load_3d_pair(&tmB, bar, sa + A_STAGE, c * BK, nt * x.bn + rank * (x.bn / 2), 0);
                 }
             }
-            // drain: wait for every load still in flight, of both CTAs (at most one per stage)
+            // both CTAs learn of the other's count (compared behind the cluster barrier below)
+            issued[rank] = it;
+            store_cluster(map_to_rank(const_cast<uint32_t *>(issued) + rank, rank ^ 1), it);
+            // drain: wait for the loads still in flight, of both CTAs (at most one per stage)
             if (rank == 0) {
                 const uint32_t first = it > (uint32_t)STAGES ? it - STAGES : 0;
                 for (uint32_t j = first; j < it; ++j) {
@@ -472,7 +476,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
     pdl_launch();
     tc_fence_before();
     __syncthreads();
+    // the commits signal CTA 1's barriers too; it stays until the last of them has
+    if (rank == 1 && warp == 1) mbar_wait(mma_done, 0, tmo, nullptr);
+    __syncwarp();
     cluster_sync();   // neither CTA frees its tensor memory or leaves while the other may still use it
+    if (issued[1] > issued[0]) {
+        // After a wait that ran out CTA 1 may have loaded a stage more than CTA 0: those loads complete
+        // on CTA 0's barrier, which nobody has armed for them, and CTA 1 must not leave before they do.
+        if (rank == 0 && threadIdx.x == 0)
+            for (uint32_t j = issued[0]; j < issued[1]; ++j) {
+                mbar_arrive_expect_tx(&full[j % STAGES], stage_bytes);
+                mbar_wait(&full[j % STAGES], (j / STAGES) & 1, tmo, nullptr);
+            }
+        __syncwarp();
+        __syncthreads();
+        cluster_sync();
+    }
     tc_fence_after();
     if (warp == 1) tmem_dealloc_pair(tmem_base, TMEM_COLS);
 }
