@@ -3,7 +3,7 @@
 // The GEMM of the TTGT reformulation (Section 2, C_p[i,k] = A_p[i,j] * B_p[j,k]; Section 6
 // "GEMM optimizations" for the blocking of C into tiles and of K into panels) with FP32 (or
 // FP64) operands carried as two FP16 parts x * 2^(14-e) = h + l (written by the split pre-pass in
-// [plane][row][K] order, K contiguous; see split2 in split.cuh).
+// [plane][row][K] order, K contiguous; see HalfScale in split.cuh).
 //
 // Numerics.  Three products are kept: hh, hl and lh (ll is at most 2^-22 of the operands'
 // leading powers of two).  The tensor core's FP32 accumulation truncates, so a long K would
@@ -11,12 +11,15 @@
 // zero, its correction MMAs (2^-11 of the result) first and its two or four hh MMAs last, and the
 // epilogue warps add the chunks into FP32 register sums of two levels (round to nearest).  At
 // the end of a tile the sum is scaled by alpha * 2^(eA + eB - 28) and stored.
-// Relative 2-norm error against FP64, K = 64 / 576 / 1633 / 12288, and what three fixed-point
-// bfloat16 parts with six products gave (whose parts are relative to the largest element):
-//   uniform in [-1, 1)   0.98 1.13 1.23 1.63e-7   (1.30 1.33 1.32 1.5e-7)
-//   uniform in +-0.7     1.09 1.22 1.31 1.69e-7   (2.2e-7)
-//   normal               1.05 1.19 1.29 1.68e-7   (18e-7)
-// Chunks of 64 throughout: 1.26 .. 1.63e-7 (uniform); one level of sums: 2.8e-7 at K = 12288.
+// Relative 2-norm error against FP64, measured (M = N = 1024, K = 64 / 576 / 1633 / 4800 / 12288), and in
+// brackets that of three fixed-point bfloat16 parts with six products, whose parts are relative to the
+// largest element and whose leading products sum exactly:
+//   uniform in [-1, 1)   0.87 1.02 1.13 1.45 1.56e-7   (1.10 1.11 1.16 1.24 3.99e-7; 1.2 to 4.0 by the seed)
+//   uniform in +-0.7     1.10 1.23 1.32 1.59 1.70e-7   (2.17 2.19 2.21 2.26 2.32e-7)
+//   normal               1.06 1.19 1.29 1.57 1.68e-7   (18.3 18.4 18.4 18.4 18.4e-7)
+//   uniform in [0, 1)    0.91 0.93 0.94 1.91 1.92e-7   (0.34 0.31 0.34 0.64 0.81e-7)
+// So operands of one sign, whose chunks are all truncated the same way, lose by it.  Chunks of 32 beyond
+// K = 4096 too (plan option kc): uniform 1.28 and 1.47e-7, one sign 1.02 and 1.09e-7, 15 to 30 % more time.
 //
 // GB300 form: one persistent pair of CTAs (cluster of two, 512 threads each) per two SMs, the
 // pair's output tile 256 x bn (bn = 48 .. 192, chosen by split_schedule):
@@ -32,8 +35,8 @@
 //                and at the end of the tile stores through the output's strides (the output
 //                permutation of TTGT folded in; through shared memory where its runs lie along N)
 //   3-stage shared-memory ring (56 KB per stage and CTA at bn = 192).
-// What bounds it: the power cap at large sizes.  M = N = K = 12288: 7.0 ms = 1.6 PFLOP/s of MMA
-// (six bf16 products: 10.7-10.9 ms); at middle sizes the hand-over of an accumulator per chunk (see NBUF).
+// What bounds it: the power cap at large sizes.  M = N = K = 12288: 6.8 to 7.4 ms by the box = 1.5 to
+// 1.6 PFLOP/s of MMA (six bf16 products: 10.7-10.9 ms); at middle sizes the hand-over of an accumulator per chunk (see NBUF).
 // Why pairs: with one CTA per 128 x 256 tile a stage reads 144 KB of operands from shared memory
 // and fills 96 KB per 1536 MMA cycles, 160 bytes per clock against the SM's 128; in a pair each
 // CTA holds half of B (bn = 192: 84 + 56 KB per 1152 cycles, 121).  Tiles of 240 and 256 columns ran

@@ -97,7 +97,7 @@ struct XposeParams {
     Radix u, v, r;
     const void *in;
     void *out;
-    int64_t out_plane;             // split pre-pass: element distance between the 3 planes
+    int64_t out_plane;             // split pre-pass: element distance between the planes
     const void *slots;             // split pre-pass: n_slots 8-byte words, the bits of max |x| of a
     uint32_t n_slots;              // part of the operand each
     void *scale_out;               // split pre-pass: word that receives the bits of their maximum

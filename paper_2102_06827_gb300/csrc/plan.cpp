@@ -1109,8 +1109,9 @@ comet_status_t build_plan(const char *expr, const comet_extent_t *extents, int n
             bk = (size_t)emu_partial_bytes(sch);
         }
         if (st.kernel == KK_GEMM_SPLIT) {
-            // tile width and K slices (split_schedule); the step's room is never less than the three planes
-            // per operand that were kept before
+            // Tile width and K slices (split_schedule).  The step's room is never less than three planes per
+            // operand take, although it holds two: so the plans that the no-alloc entry refuses stay the same,
+            // and the slices' partial sums have room without a larger workspace.
             least = align((size_t)6 * rows_a * st.kpad) + align((size_t)6 * rows_b * st.kpad);
             st.want_ksplit = opts.ksplit > 0 ? (uint32_t)opts.ksplit : 0;
             const SplitSchedule sch = split_schedule((uint64_t)rows_a, (uint64_t)rows_b, (uint64_t)Kx, 76,
