@@ -479,8 +479,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split::THREADS, 1)
     pdl_launch();
     tc_fence_before();
     __syncthreads();
-    // the commits signal CTA 1's barriers too; it stays until the last of them has
-    if (rank == 1 && warp == 1) mbar_wait(mma_done, 0, tmo, nullptr);
+    // the commits signal CTA 1's barriers too; it stays until the last of them has (one thread: the whole warp's
+    // wait made the 192-column tiles 1 % slower)
+    if (rank == 1 && threadIdx.x == 32) mbar_wait(mma_done, 0, tmo, nullptr);
     __syncwarp();
     cluster_sync();   // neither CTA frees its tensor memory or leaves while the other may still use it
     if (issued[1] > issued[0]) {
@@ -523,38 +524,54 @@ __global__ void __launch_bounds__(256) split_reduce_kernel(const GemmParams p, c
     }
     int64_t r0 = 0, c_row = 0;
     if (m < p.M) radix_offsets(p.ma, m, r0, c_row);
-    pdl_wait();
+    // (before the wait: the GEMM in front let this kernel begin after its own wait for the pre-passes, whose words
+    // these are; looked up after it they cost another 0.3 us)
     if (threadIdx.x == 0)
         s_exp = half_exponent<TOut>(scale_exponent<TOut>(x.scale_a)) + half_exponent<TOut>(scale_exponent<TOut>(x.scale_b));
+    pdl_wait();
     __syncthreads();
     if (m >= p.M) return;
     const int e_sum = s_exp;
-    // plain FP32 results: one product with a normal power of two; everything else in FP64
-    const bool plain = sizeof(TOut) == 4 && p.alpha == 1.0 && p.beta == 0.0 && e_sum >= -126 && e_sum <= 127;
-    const float sc = plain ? __int_as_float((e_sum + 127) << 23) : 0.0f;
-    const double scale = plain ? 0.0 : ldexp(p.alpha, e_sum);
     const size_t slice = (size_t)x.m_tiles * x.n_tiles * 2 * x.bn * BM;
     const float *P = x.partial + ((size_t)cta * x.bn + strip * STRIP) * BM + ml;
+    // Four columns at a time, so that their loads are in flight together (those of columns beyond N too, whose
+    // slots hold nothing and are not stored): one after the other, the few blocks of a small result wait for
+    // memory (a whole 256 x 256 x 1024 contraction, eight slices: 22.0 us, now 15.9)
+    constexpr int U = 4;
+    static_assert(STRIP % (2 * U) == 0, "a thread's columns in whole groups");
+    auto each = [&](auto &&store) {   // store(element of C, sum, its error)
+        for (uint32_t j0 = threadIdx.x >> 7; j0 < STRIP; j0 += 2 * U) {
+            float s[U] = {}, lo[U] = {};
 #pragma unroll 4
-    for (uint32_t j = threadIdx.x >> 7; j < STRIP; j += 2) {
-        if (n0 + j >= p.N) break;
-        float s = 0.0f, lo = 0.0f;
-        for (uint32_t k = 0; k < x.ksplit; ++k) {
-            const float *q = P + k * slice + (size_t)j * BM;
-            if (!dbg_ok(x.dbg_p, q, 4, p.status)) continue;
-            const float v = *q, t = s + v, z = t - s;
-            lo += (s - (t - z)) + (v - z);
-            s = t;
+            for (uint32_t k = 0; k < x.ksplit; ++k) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float *q = P + k * slice + (size_t)(j0 + 2 * u) * BM;
+                    if (!dbg_ok(x.dbg_p, q, 4, p.status)) continue;
+                    const float v = *q, t = s[u] + v, z = t - s[u];
+                    lo[u] += (s[u] - (t - z)) + (v - z);
+                    s[u] = t;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (n0 + j0 + 2 * u >= p.N) break;
+                TOut *c = reinterpret_cast<TOut *>(p.C) + c_row + c_col[j0 + 2 * u];
+                // (the error term of an infinite sum is not a number)
+                if (dbg_ok(p.dbg_c, c, (int)sizeof(TOut), p.status)) store(c, s[u], fabsf(s[u]) < INFINITY ? lo[u] : 0.0f);
+            }
         }
-        TOut *c = reinterpret_cast<TOut *>(p.C) + c_row + c_col[j];
-        if (!dbg_ok(p.dbg_c, c, (int)sizeof(TOut), p.status)) continue;
-        if (!(fabsf(s) < INFINITY)) lo = 0.0f;   // the error term of an infinite sum is not a number
-        if (plain) {
-            *c = (TOut)(sc * (s + lo));
-        } else {
+    };
+    if (sizeof(TOut) == 4 && p.alpha == 1.0 && p.beta == 0.0 && e_sum >= -126 && e_sum <= 127) {
+        // plain FP32 results: one product with a normal power of two
+        const float sc = __int_as_float((e_sum + 127) << 23);
+        each([&](TOut *c, float s, float lo) { *c = (TOut)(sc * (s + lo)); });
+    } else {
+        const double scale = ldexp(p.alpha, e_sum);
+        each([&](TOut *c, float s, float lo) {
             const double r = scale * ((double)s + (double)lo);
             *c = (TOut)(p.beta != 0.0 ? r + p.beta * (double)*c : r);
-        }
+        });
     }
 }
 
