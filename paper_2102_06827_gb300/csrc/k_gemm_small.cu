@@ -14,7 +14,7 @@
 // in all, nothing beside a row's and a column's largest elements if their product reaches K 2^-123.  A tile
 // with a sum too small to rule that out (a zero too) looks its rows' and columns' largest elements up, and
 // where a pair's product lies below that line runs again with each of them scaled to about one.  At M = N = K =
-// 192: 6.0 us, 9.3 with zeros in every tile, 15.3 where all products are below the line.
+// 192: 6.0 us, 8.8 with zeros in every tile, 14.6 where all products are below the line.
 //
 // Blocking: a 16 x 16 output tile per block of 256 threads, which also split K four ways (64
 // threads with 2 x 2 outputs each per quarter): at M = N = K = 192 there are 144 tiles, about one for
@@ -126,8 +126,9 @@ __device__ __forceinline__ void multiply_chunk(const float *sm, int nk, float (&
     }
 }
 
-// The quarters' sums, [quarter][column][row], then output (t % 16, t / 16) per thread: sum and its error
-__device__ __forceinline__ float2 add_quarters(float *sm, const float (&s)[2][2], const float (&c)[2][2]) {
+// The quarters' sums, [quarter][column][row], then output (t % 16, t / 16) per thread: sum and its error.
+// *any: whether `flag` is set in some thread of the block.
+__device__ __forceinline__ float2 add_quarters(float *sm, const float (&s)[2][2], const float (&c)[2][2], bool flag, bool *any) {
     using namespace sg;
     const int t = threadIdx.x, kq = t >> 6, q = t & 63, tm = (q & 7) * 2, tn = (q >> 3) * 2;
     __syncthreads();
@@ -136,7 +137,7 @@ __device__ __forceinline__ float2 add_quarters(float *sm, const float (&s)[2][2]
     for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j) part[(kq * TM + tn + j) * TM + tm + i] = make_float2(s[i][j], c[i][j]);
-    __syncthreads();
+    *any = __syncthreads_or(flag);
     float hi = 0.0f, lo = 0.0f;
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
@@ -149,10 +150,9 @@ __device__ __forceinline__ float2 add_quarters(float *sm, const float (&s)[2][2]
 }
 
 // A tile with a sum so small that products may have lost bits below the range (see above): the sum and error
-// of this thread's output again, as 2^-e_sum of the result, or v as it was.  The whole block calls
-// it; not inlined, so that the ordinary tile's code stays as short as it was.
+// of this thread's output again, as 2^-e_sum of the result, or v as it was.  The whole block calls it.
 template <bool AK, bool BK>
-__device__ __noinline__ float2 sum_scaled(const GemmParams &p, Offsets &o, float *sm, int rows, int cols, float2 v, int *e_sum) {
+__device__ __forceinline__ float2 sum_scaled(const GemmParams &p, Offsets &o, float *sm, int rows, int cols, float2 v, int *e_sum) {
     using namespace sg;
     const int t = threadIdx.x, r = t & 15, n = t >> 4;
     // the rows' and columns' largest finite magnitudes, eight threads each
@@ -187,7 +187,8 @@ __device__ __noinline__ float2 sum_scaled(const GemmParams &p, Offsets &o, float
         multiply_chunk<AK, BK>(sm, nk, s, c);
     }
     *e_sum = scale(ea) + scale(eb);
-    return add_quarters(sm, s, c);
+    bool any;
+    return add_quarters(sm, s, c, false, &any);
 }
 
 template <bool AK, bool BK>
@@ -213,12 +214,22 @@ __global__ void __launch_bounds__(sg::T) gemm_small_kernel(const __grid_constant
         const int nk = load_chunk<AK, BK>(p, o, sm, k0, rows, cols);
         multiply_chunk<AK, BK>(sm, nk, s, c);
     }
-    float2 v = add_quarters(sm, s, c);
+    // Whether a quarter's sum is as small as K products of less than K 2^-123.  (The vote is the barrier that the
+    // quarters meet at anyway; behind a barrier of its own, and with sum_scaled not inlined, 64 registers: 12 to 15 %
+    // more at the upper end of this kernel's sizes.)
+    bool tiny = false;
+    const int q = t & 63, tm = (q & 7) * 2, tn = (q >> 3) * 2;
+    const float line = (float)p.K * (float)p.K * 0x1p-123f;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) tiny |= tm + i < rows && tn + j < cols && fabsf(s[i][j]) < line;
+    tiny &= 2 * (t >> 6) < p.K;   // (a quarter without a K value says nothing)
+    int e_sum = 0;   // v carries 2^-e_sum of the result
+    float2 v = add_quarters(sm, s, c, tiny, &tiny);
+    if (__builtin_expect(tiny, 0)) v = sum_scaled<AK, BK>(p, o, sm, rows, cols, v, &e_sum);
     const int r = t & 15, n = t >> 4;
     const bool in = r < rows && n < cols;
-    int e_sum = 0;   // v carries 2^-e_sum of the result
-    if (__syncthreads_or(in && fabsf(v.x + v.y) < (float)p.K * (float)p.K * 0x1p-123f))
-        v = sum_scaled<AK, BK>(p, o, sm, rows, cols, v, &e_sum);
     pdl_launch();   // (before the quarters meet it costs 2 us on M = N = K = 192: the next grid's blocks crowd in)
     if (!in) return;
     double sum = (double)v.x + (double)v.y;
