@@ -81,9 +81,9 @@ struct Step {
     uint32_t chunk = 0;          // split GEMM: K values per accumulation chunk
     size_t ws_ksplit = 0;        // workspace offset of the slices' FP32 partials
     size_t ksplit_bytes = 0;     // their size
-    uint32_t tail_tiles = 0, tail_slices = 1;   // description: what 128 x 256 tiles leave over after
-                                                // whole waves of 152 SMs, at most half of them, and
-                                                // the K slices of it that would fill them
+    uint32_t tail_tiles = 0, tail_slices = 1;   // Plan.info only, no kernel has such a tail: what 128 x 256
+                                                // tiles leave over after whole waves of 152 SMs, at most
+                                                // half of them, and the K slices that would fill them
     // precomputed parameter blocks (pointers filled at launch)
     GemmParams gemm;             // for both GEMM kernels (offsets in elements)
     XposeParams pre_a, pre_b;    // split pre-passes (A then B operand)
